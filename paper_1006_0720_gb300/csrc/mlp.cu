@@ -7,8 +7,8 @@
 // Inputs per node: <U>, <V>, <W>, <uu>, <vv>, <ww>, <uv>, <uw>, <vw>,
 // <omega>, wall distance; outputs wp_ij.  Both standardized with stored
 // means and scales.  Matrix products on the tensor cores (mma.sync
-// m16n8k16, BF16 x BF16 -> FP32); the weight gradients, a reduction over
-// the batch, in FP32 in a fixed order (deterministic).
+// m16n8k16, BF16 x BF16 -> FP32), the weight gradients' sums over the batch
+// too, in a fixed order (deterministic).
 // Rounding points (shared with the CPU check): the standardized input, the
 // weights, every hidden activation and every back-propagated gradient are
 // rounded to BF16 before they enter a product.
@@ -75,10 +75,6 @@ __device__ __forceinline__ void mma_bf16(float c[4], const uint32_t a[4], uint32
 }
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float z) {
-  return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
-}
-
 // One layer for a warp's 16 rows: C[16][8*NT] = A[16][16*KT] * W^T, with A
 // in fragment registers (KT k-tiles) and W [N][K] row-major in shared memory
 // (ld = padded K).
@@ -111,9 +107,12 @@ __device__ __forceinline__ void c_to_a(const float (&C)[NT][4], uint32_t (&A)[NT
   }
 }
 
+// row strides (BF16) of 16- and 64-wide arrays in shared memory
+constexpr int kLd16 = 24, kLd64 = 72;
+
 // Standardized input rows -> A fragments of layer 0 (K padded to 16).
 __device__ __forceinline__ void load_input(const float* __restrict__ X, int64_t n, int64_t row0,
-                                           const float* norm, uint32_t (&A)[1][4], __nv_bfloat16* a0s /*[16][16] or null*/) {
+                                           const float* norm, uint32_t (&A)[1][4], __nv_bfloat16* a0s /*16 rows of kLd16, or null*/) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   float v[2][4];
 #pragma unroll
@@ -135,16 +134,40 @@ __device__ __forceinline__ void load_input(const float* __restrict__ X, int64_t 
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int row = g + ((q & 1) ? 8 : 0), col = 2 * t + ((q & 2) ? 8 : 0);
-      *reinterpret_cast<uint32_t*>(a0s + row * 16 + col) = A[0][q];
+      *reinterpret_cast<uint32_t*>(a0s + row * kLd16 + col) = A[0][q];
     }
   }
 }
 
+// Weights in shared memory: rows padded by 8 BF16 (strides of 24 and 72), so
+// that the eight rows of a fragment load and the eight rows of an ldmatrix
+// fall into different banks (unpadded 128-byte rows all start in bank 0: an
+// 8-way conflict on every fragment).  The order is W0 W1 W2 W3 (the forward
+// pass) then WT3 WT2 WT1 (the backward pass).
+__host__ __device__ constexpr int kSmW_(int l) { return l == 0 ? 0 : l == 1 ? 1536 : l == 2 ? 6144 : 10752; }
+__host__ __device__ constexpr int kSmWT_(int l) { return l == 3 ? 11904 : l == 2 ? 13440 : 18048; }
+constexpr int kSmFwd = 11904, kSmAll = 22656;
+
+template <int ROW>  // ROW real BF16 per row (16 or 64), 16 bytes per access
+__device__ __forceinline__ void stage_rows(const __nv_bfloat16* __restrict__ src, __nv_bfloat16* dst, int rows) {
+  constexpr int kPer = ROW / 8, kLd = ROW == 16 ? kLd16 : kLd64;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < rows * kPer; i += blockDim.x)
+    *reinterpret_cast<uint4*>(dst + (i / kPer) * kLd + (i % kPer) * 8) = __ldg(reinterpret_cast<const uint4*>(src) + i);
+}
+
 __device__ __forceinline__ void stage_weights(const __nv_bfloat16* __restrict__ wb, const float* __restrict__ bias,
                                               const float* __restrict__ norm, __nv_bfloat16* s_w, float* s_b,
-                                              float* s_norm, int n_wb) {
-  for (int i = threadIdx.x; i < n_wb / 2; i += blockDim.x)
-    reinterpret_cast<uint32_t*>(s_w)[i] = reinterpret_cast<const uint32_t*>(wb)[i];
+                                              float* s_norm, bool backward) {
+  stage_rows<16>(wb + kOffWb_(0), s_w + kSmW_(0), 64);
+  stage_rows<64>(wb + kOffWb_(1), s_w + kSmW_(1), 64);
+  stage_rows<64>(wb + kOffWb_(2), s_w + kSmW_(2), 64);
+  stage_rows<64>(wb + kOffWb_(3), s_w + kSmW_(3), 16);
+  if (backward) {
+    stage_rows<16>(wb + kOffWT_(3), s_w + kSmWT_(3), 64);
+    stage_rows<64>(wb + kOffWT_(2), s_w + kSmWT_(2), 64);
+    stage_rows<64>(wb + kOffWT_(1), s_w + kSmWT_(1), 64);
+  }
   for (int i = threadIdx.x; i < kNBias; i += blockDim.x) s_b[i] = bias[i];
   for (int i = threadIdx.x; i < 64; i += blockDim.x) s_norm[i] = norm[i];
   __syncthreads();
@@ -154,9 +177,9 @@ __device__ __forceinline__ void stage_weights(const __nv_bfloat16* __restrict__ 
 __global__ void __launch_bounds__(kThreads) k_mlp_fwd(const __nv_bfloat16* __restrict__ wb,
                                                        const float* __restrict__ bias, const float* __restrict__ norm,
                                                        const float* __restrict__ X, int64_t n, float* __restrict__ Y) {
-  __shared__ __align__(16) __nv_bfloat16 s_w[10240];
+  __shared__ __align__(16) __nv_bfloat16 s_w[kSmFwd];
   __shared__ float s_b[kNBias], s_norm[64];
-  stage_weights(wb, bias, norm, s_w, s_b, s_norm, kOffWT_(0));
+  stage_weights(wb, bias, norm, s_w, s_b, s_norm, false);
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5;
   const int64_t chunks = (n + 15) / 16;
   for (int64_t c = (int64_t)blockIdx.x * 4 + w; c < chunks; c += (int64_t)gridDim.x * 4) {
@@ -165,7 +188,7 @@ __global__ void __launch_bounds__(kThreads) k_mlp_fwd(const __nv_bfloat16* __res
     load_input(X, n, row0, s_norm, A0, nullptr);
     float C[8][4];
     uint32_t A[4][4];
-    layer_mma<1, 8>(A0, s_w + kOffWb_(0), 16, C);
+    layer_mma<1, 8>(A0, s_w + kSmW_(0), kLd16, C);
 #pragma unroll
     for (int j = 0; j < 8; ++j)
 #pragma unroll
@@ -173,7 +196,7 @@ __global__ void __launch_bounds__(kThreads) k_mlp_fwd(const __nv_bfloat16* __res
     c_to_a<8>(C, A);
 #pragma unroll
     for (int l = 1; l <= 2; ++l) {
-      layer_mma<4, 8>(A, s_w + kOffWb_(l), 64, C);
+      layer_mma<4, 8>(A, s_w + kSmW_(l), kLd64, C);
 #pragma unroll
       for (int j = 0; j < 8; ++j)
 #pragma unroll
@@ -181,7 +204,7 @@ __global__ void __launch_bounds__(kThreads) k_mlp_fwd(const __nv_bfloat16* __res
       c_to_a<8>(C, A);
     }
     float O[2][4];
-    layer_mma<4, 2>(A, s_w + kOffWb_(3), 64, O);
+    layer_mma<4, 2>(A, s_w + kSmW_(3), kLd64, O);
 #pragma unroll
     for (int j = 0; j < 2; ++j)
 #pragma unroll
@@ -196,27 +219,39 @@ __global__ void __launch_bounds__(kThreads) k_mlp_fwd(const __nv_bfloat16* __res
 
 // Training pass: forward, backward, per-CTA partial gradients of the mean
 // squared error (over the batch and the 9 standardized outputs).
+//
+// One CTA takes 64 rows at a time, a warp 16 of them.  The weight gradients
+// dW_l = dz_l^T a_l are products too (M = outputs, N = inputs, K = the 64
+// rows) and run on the tensor cores from the BF16 operands that the forward
+// and backward passes leave in shared memory: warp w owns 16 output rows of
+// W0, W1 and W2 and 16 input columns of W3, reads both operands transposed
+// (ldmatrix.trans) and adds each block's FP32 sums to its registers; a
+// bias gradient is the same product with a column of ones.  Each block's
+// sum is formed first and then added, and CTAs are summed in order, so the
+// result is deterministic.  At 8,192 rows (128 CTAs) the pass took 257 us
+// with scalar loops over the rows (9,673 sums of 64 products per block on
+// 128 threads) and unpadded weight rows; a whole gradient call went from 292
+// to 53 us with this form.  What bounds it now is the latency of one
+// block's chain of layers.
 struct TrainSmem {
-  __nv_bfloat16 w[kNWb];              // W_l and WT_l
+  __nv_bfloat16 w[kSmAll];            // W_l and WT_l
+  __nv_bfloat16 a0[kRows][kLd16];     // layer inputs (BF16)
+  __nv_bfloat16 a1[kRows][kLd64], a2[kRows][kLd64], a3[kRows][kLd64];
+  __nv_bfloat16 d0[kRows][kLd64], d1[kRows][kLd64], d2[kRows][kLd64], d3[kRows][kLd16];  // dz_l (BF16)
+  float4 gp[3][8][kThreads];          // gelu'(z_l) of the thread's own fragment entries
   float b[kNBias];
   float norm[64];
-  __nv_bfloat16 a0[kRows][16];        // layer inputs (BF16)
-  __nv_bfloat16 a1[kRows][64], a2[kRows][64], a3[kRows][64];
-  float z0[kRows][64], z1[kRows][64], z2[kRows][64];  // pre-activations
-  __nv_bfloat16 d0[kRows][64], d1[kRows][64], d2[kRows][64], d3[kRows][16];  // dz_l (BF16)
-  float acc[kNParam];                 // this CTA's gradient
   float loss[4];
 };
 
-__device__ __forceinline__ void store_c(const float (&C)[8][4], float (*z)[64], int rbase) {
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-#pragma unroll
-  for (int j = 0; j < 8; ++j)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) z[rbase + g + ((e & 2) ? 8 : 0)][j * 8 + 2 * t + (e & 1)] = C[j][e];
+// gelu(z) and gelu'(z) with the error function taken once.
+__device__ __forceinline__ float gelu_both(float z, float& grad) {
+  const float c = 0.5f * (1.0f + erff(z * 0.70710678118654752f));
+  grad = c + z * 0.39894228040143268f * expf(-0.5f * z * z);
+  return z * c;
 }
 
-__device__ __forceinline__ void store_a(const uint32_t (&A)[4][4], __nv_bfloat16 (*a)[64], int rbase) {
+__device__ __forceinline__ void store_a(const uint32_t (&A)[4][4], __nv_bfloat16 (*a)[kLd64], int rbase) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
   for (int q = 0; q < 4; ++q)
@@ -227,6 +262,79 @@ __device__ __forceinline__ void store_a(const uint32_t (&A)[4][4], __nv_bfloat16
     }
 }
 
+__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], const __nv_bfloat16* p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a));
+}
+
+// acc[i] += sum over the block's 64 rows of dz[row][m0 + .] a[row][n0 + 8 i + .]
+// for NT n-tiles (an even number), and with BIAS acc_b += the row sums of dz.
+// dz and a are row-major [64][ld] (K along the rows): both fragments come
+// from transposed 8 x 8 loads.  A (16 outputs x 16 rows): matrices (rows 0-7,
+// m 0-7), (0-7, 8-15), (8-15, 0-7), (8-15, 8-15) -> a0, a1, a2, a3.  B (16 rows
+// x 16 columns): (rows 0-7, n 0-7), (8-15, 0-7), (0-7, 8-15), (8-15, 8-15).
+template <int NT, bool BIAS>
+__device__ __forceinline__ void grad_mma(const __nv_bfloat16* dz, int ldd, int m0, const __nv_bfloat16* a, int lda,
+                                         int n0, float (&acc)[NT][4], float (&acc_b)[2]) {
+  const int lane = threadIdx.x & 31, q = lane >> 3, r = lane & 7;
+  uint32_t A[4][4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    ldsm_x4_t(A[k], dz + (16 * k + r + ((q & 2) ? 8 : 0)) * ldd + m0 + ((q & 1) ? 8 : 0));
+#pragma unroll
+  for (int i = 0; i < NT; i += 2) {
+    float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      uint32_t B[4];
+      ldsm_x4_t(B, a + (16 * k + r + ((q & 1) ? 8 : 0)) * lda + n0 + 8 * i + ((q & 2) ? 8 : 0));
+      mma_bf16(c0, A[k], B[0], B[1]);
+      mma_bf16(c1, A[k], B[2], B[3]);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      acc[i][e] += c0[e];
+      acc[i + 1][e] += c1[e];
+    }
+  }
+  if (BIAS) {
+    float c[4] = {0.f, 0.f, 0.f, 0.f};
+    const uint32_t ones = 0x3F803F80u;  // two BF16 ones
+#pragma unroll
+    for (int k = 0; k < 4; ++k) mma_bf16(c, A[k], ones, ones);
+    acc_b[0] += c[0];  // output g; every column holds the same sum
+    acc_b[1] += c[2];  // output g + 8
+  }
+}
+
+// One hidden layer's activation: bias, gelu and gelu' (kept for the way back).
+__device__ __forceinline__ void activate(float (&C)[8][4], const float* b, float4 (*gp)[kThreads]) {
+  const int t = threadIdx.x & 3;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    float4 d;
+    const float b0 = b[j * 8 + 2 * t], b1 = b[j * 8 + 2 * t + 1];
+    C[j][0] = gelu_both(C[j][0] + b0, d.x);
+    C[j][1] = gelu_both(C[j][1] + b1, d.y);
+    C[j][2] = gelu_both(C[j][2] + b0, d.z);
+    C[j][3] = gelu_both(C[j][3] + b1, d.w);
+    gp[j][threadIdx.x] = d;
+  }
+}
+
+__device__ __forceinline__ void times_gp(float (&C)[8][4], const float4 (*gp)[kThreads]) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const float4 d = gp[j][threadIdx.x];
+    C[j][0] *= d.x;
+    C[j][1] *= d.y;
+    C[j][2] *= d.z;
+    C[j][3] *= d.w;
+  }
+}
+
 __global__ void __launch_bounds__(kThreads) k_mlp_train(const __nv_bfloat16* __restrict__ wb,
                                                          const float* __restrict__ bias, const float* __restrict__ norm,
                                                          const float* __restrict__ X, const float* __restrict__ Yt,
@@ -234,60 +342,35 @@ __global__ void __launch_bounds__(kThreads) k_mlp_train(const __nv_bfloat16* __r
                                                          float* __restrict__ loss_part) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
-  stage_weights(wb, bias, norm, S.w, S.b, S.norm, kNWb);
-  for (int i = threadIdx.x; i < kNParam; i += kThreads) S.acc[i] = 0.f;
-  if (threadIdx.x < 4) S.loss[threadIdx.x] = 0.f;
-  __syncthreads();
+  stage_weights(wb, bias, norm, S.w, S.b, S.norm, true);
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5;
   const float inv_count = 1.0f / (float)(n * kOut);
   float my_loss = 0.f;
+  float g0[2][4] = {}, g1[8][4] = {}, g2[8][4] = {}, g3[2][4] = {};  // this warp's weight gradients
+  float h0[2] = {}, h1[2] = {}, h2[2] = {}, h3[2] = {};              // and bias gradients
   const int64_t blocks = (n + kRows - 1) / kRows;
   for (int64_t blk = blockIdx.x; blk < blocks; blk += gridDim.x) {
     const int64_t row0 = blk * kRows + w * 16;
     const int rb = w * 16;
-    // ---- forward, keeping layer inputs and pre-activations
+    // ---- forward, keeping layer inputs and gelu'
     uint32_t A0[1][4];
     load_input(X, n, row0, S.norm, A0, &S.a0[rb][0]);
     float C[8][4];
     uint32_t A[4][4];
-    layer_mma<1, 8>(A0, S.w + kOffWb_(0), 16, C);
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) C[j][e] += S.b[kOffBias_(0) + j * 8 + 2 * t + (e & 1)];
-    store_c(C, S.z0, rb);
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) C[j][e] = gelu(C[j][e]);
+    layer_mma<1, 8>(A0, S.w + kSmW_(0), kLd16, C);
+    activate(C, S.b + kOffBias_(0), S.gp[0]);
     c_to_a<8>(C, A);
     store_a(A, S.a1, rb);
-    layer_mma<4, 8>(A, S.w + kOffWb_(1), 64, C);
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) C[j][e] += S.b[kOffBias_(1) + j * 8 + 2 * t + (e & 1)];
-    store_c(C, S.z1, rb);
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) C[j][e] = gelu(C[j][e]);
+    layer_mma<4, 8>(A, S.w + kSmW_(1), kLd64, C);
+    activate(C, S.b + kOffBias_(1), S.gp[1]);
     c_to_a<8>(C, A);
     store_a(A, S.a2, rb);
-    layer_mma<4, 8>(A, S.w + kOffWb_(2), 64, C);
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) C[j][e] += S.b[kOffBias_(2) + j * 8 + 2 * t + (e & 1)];
-    store_c(C, S.z2, rb);
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) C[j][e] = gelu(C[j][e]);
+    layer_mma<4, 8>(A, S.w + kSmW_(2), kLd64, C);
+    activate(C, S.b + kOffBias_(2), S.gp[2]);
     c_to_a<8>(C, A);
     store_a(A, S.a3, rb);
     float O[2][4];
-    layer_mma<4, 2>(A, S.w + kOffWb_(3), 64, O);
+    layer_mma<4, 2>(A, S.w + kSmW_(3), kLd64, O);
     // ---- output gradient dL/dy = 2 (y - t) / (n 9), rows past n and padded columns 0
     float D[2][4];
 #pragma unroll
@@ -318,55 +401,25 @@ __global__ void __launch_bounds__(kThreads) k_mlp_train(const __nv_bfloat16* __r
     }
     // ---- back through layers 3..1: da = dz W (B operand from WT), dz = da * gelu'(z)
     float Cd[8][4];
-    layer_mma<1, 8>(G3, S.w + kOffWT_(3), 16, Cd);  // WT3 [64][16]: da2 [16][64]
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        Cd[j][e] *= gelu_grad(S.z2[rb + g + ((e & 2) ? 8 : 0)][j * 8 + 2 * t + (e & 1)]);
+    layer_mma<1, 8>(G3, S.w + kSmWT_(3), kLd16, Cd);  // WT3 [64][16]: da2 [16][64]
+    times_gp(Cd, S.gp[2]);
     uint32_t G[4][4];
     c_to_a<8>(Cd, G);
     store_a(G, S.d2, rb);
-    layer_mma<4, 8>(G, S.w + kOffWT_(2), 64, Cd);
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        Cd[j][e] *= gelu_grad(S.z1[rb + g + ((e & 2) ? 8 : 0)][j * 8 + 2 * t + (e & 1)]);
+    layer_mma<4, 8>(G, S.w + kSmWT_(2), kLd64, Cd);
+    times_gp(Cd, S.gp[1]);
     c_to_a<8>(Cd, G);
     store_a(G, S.d1, rb);
-    layer_mma<4, 8>(G, S.w + kOffWT_(1), 64, Cd);
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        Cd[j][e] *= gelu_grad(S.z0[rb + g + ((e & 2) ? 8 : 0)][j * 8 + 2 * t + (e & 1)]);
+    layer_mma<4, 8>(G, S.w + kSmWT_(1), kLd64, Cd);
+    times_gp(Cd, S.gp[0]);
     c_to_a<8>(Cd, G);
     store_a(G, S.d0, rb);
     __syncthreads();
-    // ---- weight gradients of this block of 64 rows, FP32, fixed order
-    for (int i = threadIdx.x; i < kNParam; i += kThreads) {
-      int l = 3;
-      while (l > 0 && i < kOffW_(l)) --l;
-      float s = 0.f;
-      if (i < kOffB_(l)) {  // weight W_l[o][k]
-        const int o = (i - kOffW_(l)) / kRealK_(l), k = (i - kOffW_(l)) % kRealK_(l);
-        for (int r = 0; r < kRows; ++r) {
-          float dz, a;
-          if (l == 0) { dz = __bfloat162float(S.d0[r][o]); a = __bfloat162float(S.a0[r][k]); }
-          else if (l == 1) { dz = __bfloat162float(S.d1[r][o]); a = __bfloat162float(S.a1[r][k]); }
-          else if (l == 2) { dz = __bfloat162float(S.d2[r][o]); a = __bfloat162float(S.a2[r][k]); }
-          else { dz = __bfloat162float(S.d3[r][o]); a = __bfloat162float(S.a3[r][k]); }
-          s = fmaf(dz, a, s);
-        }
-      } else {  // bias b_l[o]
-        const int o = i - kOffB_(l);
-        for (int r = 0; r < kRows; ++r) {
-          s += __bfloat162float(l == 0 ? S.d0[r][o] : (l == 1 ? S.d1[r][o] : (l == 2 ? S.d2[r][o] : S.d3[r][o])));
-        }
-      }
-      S.acc[i] += s;
-    }
+    // ---- weight gradients of this block of 64 rows
+    grad_mma<2, true>(&S.d0[0][0], kLd64, 16 * w, &S.a0[0][0], kLd16, 0, g0, h0);
+    grad_mma<8, true>(&S.d1[0][0], kLd64, 16 * w, &S.a1[0][0], kLd64, 0, g1, h1);
+    grad_mma<8, true>(&S.d2[0][0], kLd64, 16 * w, &S.a2[0][0], kLd64, 0, g2, h2);
+    grad_mma<2, true>(&S.d3[0][0], kLd16, 0, &S.a3[0][0], kLd64, 16 * w, g3, h3);
     __syncthreads();
   }
   // loss: warp sums, then warps in order
@@ -374,24 +427,66 @@ __global__ void __launch_bounds__(kThreads) k_mlp_train(const __nv_bfloat16* __r
   for (int o = 16; o > 0; o >>= 1) my_loss += __shfl_xor_sync(0xffffffffu, my_loss, o);
   if (lane == 0) S.loss[w] = my_loss;
   __syncthreads();
-  for (int i = threadIdx.x; i < kNParam; i += kThreads) part[(int64_t)blockIdx.x * kNParam + i] = S.acc[i];
+  // fragment entry e of n-tile i: output g + 8 (e >> 1), input 8 i + 2 t + (e & 1)
+  float* P = part + (int64_t)blockIdx.x * kNParam;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const int o = g + ((e & 2) ? 8 : 0), k = 2 * t + (e & 1);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      if (8 * i + k < kIn) P[kOffW_(0) + (16 * w + o) * kIn + 8 * i + k] = g0[i][e];
+      if (o < kOut) P[kOffW_(3) + o * kHid + 16 * w + 8 * i + k] = g3[i][e];
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      P[kOffW_(1) + (16 * w + o) * kHid + 8 * i + k] = g1[i][e];
+      P[kOffW_(2) + (16 * w + o) * kHid + 8 * i + k] = g2[i][e];
+    }
+  }
+  if (t == 0) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int o = g + 8 * e;
+      P[kOffB_(0) + 16 * w + o] = h0[e];
+      P[kOffB_(1) + 16 * w + o] = h1[e];
+      P[kOffB_(2) + 16 * w + o] = h2[e];
+      if (w == 0 && o < kOut) P[kOffB_(3) + o] = h3[e];
+    }
+  }
   if (threadIdx.x == 0) loss_part[blockIdx.x] = ((S.loss[0] + S.loss[1]) + S.loss[2]) + S.loss[3];
 }
 
-// Sum the per-CTA partials in CTA order; optionally one Adam step.
-__global__ void k_mlp_reduce_adam(const float* __restrict__ part, int nparts, const float* __restrict__ loss_part,
-                                  float* __restrict__ grad, float* __restrict__ w, float* __restrict__ m,
-                                  float* __restrict__ v, float lr, float b1t, float b2t, int update,
-                                  float* __restrict__ loss_out, int64_t n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0 && loss_out) {
+// Sum the per-CTA partials; optionally one Adam step and the packed BF16
+// weights of the next pass.  Thread (x, y) of a block adds the partials y,
+// y + 8, ... of parameter x in order, then the eight sums are added in order:
+// the loads of a parameter are spread over eight threads (one thread per
+// parameter left each SM a quarter full of dependent additions).
+constexpr int kRedX = 32, kRedY = 8;
+__global__ void __launch_bounds__(kRedX* kRedY) k_mlp_reduce_adam(
+    const float* __restrict__ part, int nparts, const float* __restrict__ loss_part, float* __restrict__ grad,
+    float* __restrict__ w, float* __restrict__ m, float* __restrict__ v, float lr, float b1t, float b2t, int update,
+    __nv_bfloat16* __restrict__ wb, float* __restrict__ bias, float* __restrict__ loss_out, int64_t n) {
+  __shared__ float sums[kRedY][kRedX];
+  const int x = threadIdx.x & (kRedX - 1), y = threadIdx.x / kRedX;
+  const int i = blockIdx.x * kRedX + x;
+  if (blockIdx.x == 0 && loss_out && y == 0) {  // the first warp: lane sums, then a butterfly
     float s = 0.f;
-    for (int c = 0; c < nparts; ++c) s += loss_part[c];
-    *loss_out = s / (float)(n * kOut);
+    for (int c = x; c < nparts; c += 32) s += loss_part[c];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (x == 0) *loss_out = s / (float)(n * kOut);
   }
-  if (i >= kNParam) return;
   float s = 0.f;
-  for (int c = 0; c < nparts; ++c) s += part[(int64_t)c * kNParam + i];
+  if (i < kNParam) {
+#pragma unroll 4
+    for (int c = y; c < nparts; c += kRedY) s += __ldg(part + (int64_t)c * kNParam + i);
+  }
+  sums[y][x] = s;
+  __syncthreads();
+  if (y != 0 || i >= kNParam) return;
+  s = 0.f;
+#pragma unroll
+  for (int q = 0; q < kRedY; ++q) s += sums[q][x];
   grad[i] = s;
   if (!update) return;
   const float beta1 = 0.9f, beta2 = 0.999f, eps = 1e-8f;
@@ -399,7 +494,18 @@ __global__ void k_mlp_reduce_adam(const float* __restrict__ part, int nparts, co
   const float vi = beta2 * v[i] + (1.f - beta2) * s * s;
   m[i] = mi;
   v[i] = vi;
-  w[i] -= lr * (mi / b1t) / (sqrtf(vi / b2t) + eps);
+  const float wn = w[i] - lr * (mi / b1t) / (sqrtf(vi / b2t) + eps);
+  w[i] = wn;
+  int l = 3;
+  while (l > 0 && i < kOffW_(l)) --l;
+  if (i >= kOffB_(l)) {
+    bias[kOffBias_(l) + i - kOffB_(l)] = wn;
+  } else {  // the padding of the packed forms stays zero
+    const int rel = i - kOffW_(l), o = rel / kRealK_(l), k = rel % kRealK_(l);
+    const __nv_bfloat16 q = __float2bfloat16_rn(wn);
+    wb[kOffWb_(l) + o * kPadK_(l) + k] = q;
+    wb[kOffWT_(l) + k * kPadN_(l) + o] = q;
+  }
 }
 
 // FP32 master parameters -> packed BF16 weights (and transposes), padded biases.
@@ -611,10 +717,9 @@ static pdf_status mlp_pass(pdf_mlp* M, const float* X, const float* Y, int64_t n
     b1t = 1.f - powf(0.9f, (float)M->t);
     b2t = 1.f - powf(0.999f, (float)M->t);
   }
-  PDF_KERNEL("k_mlp_reduce_adam", st, k_mlp_reduce_adam<<<(kNParam + 255) / 256, 256, 0, st>>>(
+  PDF_KERNEL("k_mlp_reduce_adam", st, k_mlp_reduce_adam<<<(kNParam + kRedX - 1) / kRedX, kRedX * kRedY, 0, st>>>(
                                           M->part, ctas, M->loss_part, M->grad, M->w, M->m, M->v, lr, b1t, b2t, update,
-                                          loss ? M->host : nullptr, n));
-  if (update) PDF_KERNEL("k_mlp_pack", st, k_mlp_pack<<<(kNWb + 255) / 256, 256, 0, st>>>(M->w, M->wb, M->bias));
+                                          M->wb, M->bias, loss ? M->host : nullptr, n));
   if (grad_out) PDF_CUDA(cudaMemcpyAsync(grad_out, M->grad, sizeof(float) * kNParam, cudaMemcpyDefault, st));
   if (loss) {
     PDF_CUDA(cudaStreamSynchronize(st));

@@ -92,6 +92,32 @@ def test_gradients_match_the_oracle():
         assert cos > 0.9999, (name, cos)
 
 
+@pytest.mark.parametrize("n", [1, 15, 64, 65, 20000])
+def test_gradients_at_block_edges(n):
+    """One row, a partial warp, exactly one block of 64 rows, one row more,
+    and more blocks than CTAs (each CTA then sums several).  Both sides round
+    the same values to BF16, FP32 sums in another order may move one by an
+    ulp: at most 2^-8 = 3.9e-3 relative on every operand."""
+    P = _random_params(11)
+    net = pg.Mlp(0)
+    net.set_params(_flat(P), _identity_norm())
+    rng = np.random.default_rng(n)
+    X = rng.normal(size=(n, 11)).astype(np.float32)
+    Yt = rng.normal(size=(n, 9)).astype(np.float32)
+    loss, g = net.grad(torch.from_numpy(X).cuda(), torch.from_numpy(Yt).cuda())
+    ref_loss, G = OM.loss_and_grads(P, X.astype(np.float64), Yt.astype(np.float64))
+    g = _unflat(g.cpu().numpy())
+    assert abs(loss - ref_loss) < 5e-3 * ref_loss
+    for name in G:  # the weights and the biases of every layer
+        a, b = g[name].ravel(), G[name].ravel()
+        assert np.linalg.norm(a - b) < 5e-3 * np.linalg.norm(b), (name, n)
+    # a step is the same gradient through Adam: from zero moments -lr sign(g)
+    flat = _flat(g)
+    net.train_step(torch.from_numpy(X).cuda(), torch.from_numpy(Yt).cuda(), 1e-3)
+    big = np.abs(flat) > 1e-4
+    assert np.allclose((net.params()[0] - _flat(P))[big], -1e-3 * np.sign(flat[big]), rtol=0, atol=2e-6)
+
+
 def test_training_reduces_the_loss():
     rng = np.random.default_rng(5)
     n = 4096
