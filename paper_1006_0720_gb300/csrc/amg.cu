@@ -9,9 +9,10 @@
 // device at every solve (the second half of this file).
 //
 // Hierarchy (host, FP64, once): plain aggregation of the strongly connected
-// unknowns (|a_ij| >= theta sqrt(a_ii a_jj)), tentative prolongation by the
-// constant vector (the null space of the pure-Neumann matrix), smoothed
-// prolongation P = (I - w_p D^-1 A) P_tent with w_p = 4 / (3 rho(D^-1 A)),
+// unknowns (relative to each row's strongest connection), tentative
+// prolongation by the constant vector (the null space of the pure-Neumann
+// matrix), smoothed prolongation P = (I - w_p D^-1 A) P_tent with w_p =
+// 4 / (3 rho), rho a bound of the eigenvalues of D^-1 A,
 // Galerkin coarse matrices A_c = P^T A P, down to a dense coarsest matrix
 // whose inverse (for a singular matrix with constant null space the
 // regularised (A_c + mean(diag) 1 1^T / n_c)^-1, which solves every
@@ -20,18 +21,24 @@
 // One V-cycle with one damped-Jacobi sweep (W = w_s D^-1) before and after
 // the coarse correction is, per level,
 //   M^-1 b = (2 W - W A W) b + Q M_c^-1 Q^T b,   Q = (I - W A) P,
-// so the device runs two kernels per level: "down" (x = W b and
+// so the device runs two sweeps per level, "down" (x = W b and
 // b_c = Q^T b) and "up" (z = x + W (b - A x) + Q e_c), and one dense
-// matrix-vector product on the coarsest level.  The cycle is symmetric, as
+// matrix-vector product on the coarsest level (cycle.cuh: the sweeps of the
+// lower levels, or of a small system's whole solve, in one kernel).  The cycle is symmetric, as
 // the conjugate-gradient method needs.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
+#include <new>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include <cooperative_groups.h>
 
 #include "amg.cuh"
+#include "cycle.cuh"
 
 namespace pdfgb {
 
@@ -62,31 +69,135 @@ HCsr transpose(const HCsr& A) {
   return T;  // columns ascending within each row
 }
 
-// C = A B (Gustavson), columns sorted within each row.
-HCsr multiply(const HCsr& A, const HCsr& B) {
+// f(lo, hi, chunk) over chunks of the rows [0, n) on several host threads (the
+// set-up runs at the first solve of a mesh, on its critical path).  Throws
+// std::bad_alloc when a chunk did.
+constexpr int kMaxChunks = 16;
+int row_chunks(int32_t n) {
+  const int hw = (int)std::thread::hardware_concurrency();
+  return std::max(1, std::min({kMaxChunks, hw > 0 ? hw : 1, n / 1024}));
+}
+template <typename F>
+void parallel_rows(int32_t n, F f) {
+  const int c = row_chunks(n);
+  std::atomic<bool> failed{false};
+  auto run = [&](int k) {
+    try {
+      f((int32_t)((int64_t)n * k / c), (int32_t)((int64_t)n * (k + 1) / c), k);
+    } catch (...) {
+      failed = true;
+    }
+  };
+  std::thread th[kMaxChunks];
+  int started = 1;
+  for (; started < c; ++started) {
+    try {
+      th[started] = std::thread(run, started);
+    } catch (const std::system_error&) {
+      break;
+    }
+  }
+  run(0);
+  for (int k = started; k < c; ++k) run(k);  // (threads the system did not give)
+  for (int k = 1; k < started; ++k) th[k].join();
+  if (failed) throw std::bad_alloc();
+}
+
+// A matrix whose row i (n rows, m columns) is the sum of the terms that
+// terms(i, add) gives by add(column, value), in that order; columns ascending.
+template <typename F>
+HCsr row_sums(int32_t n, int32_t m, F terms) {
   HCsr C;
-  C.n = A.n;
-  C.m = B.m;
-  C.rp.assign(C.n + 1, 0);
-  std::vector<int32_t> mark(B.m, -1);
-  std::vector<double> acc(B.m, 0.0);
-  std::vector<int32_t> cols;
-  for (int32_t i = 0; i < A.n; ++i) {
-    cols.clear();
+  C.n = n;
+  C.m = m;
+  C.rp.assign(n + 1, 0);
+  std::vector<int32_t> ci[kMaxChunks];
+  std::vector<double> v[kMaxChunks];
+  parallel_rows(n, [&](int32_t lo, int32_t hi, int k) {
+    std::vector<int32_t> mark(m, -1), cols;
+    std::vector<double> acc(m, 0.0);
+    for (int32_t i = lo; i < hi; ++i) {
+      cols.clear();
+      terms(i, [&](int32_t j, double x) {
+        if (mark[j] != i) { mark[j] = i; acc[j] = 0.0; cols.push_back(j); }
+        acc[j] += x;
+      });
+      std::sort(cols.begin(), cols.end());
+      for (int32_t j : cols) { ci[k].push_back(j); v[k].push_back(acc[j]); }
+      C.rp[i + 1] = (int32_t)cols.size();
+    }
+  });
+  for (int32_t i = 0; i < n; ++i) C.rp[i + 1] += C.rp[i];
+  C.ci.reserve(C.rp[n]);
+  C.v.reserve(C.rp[n]);
+  for (int k = 0; k < kMaxChunks; ++k) {
+    C.ci.insert(C.ci.end(), ci[k].begin(), ci[k].end());
+    C.v.insert(C.v.end(), v[k].begin(), v[k].end());
+  }
+  return C;
+}
+
+// The same sums as lists: entry t of the matrix (rows rp, columns ci) is the
+// sum of weight w[k] times another array's entry id[k], off[t] <= k < off[t + 1].
+// terms(i, add) gives row i's terms by add(column, id, weight).
+struct Plan {
+  std::vector<int32_t> rp, ci, off, id;
+  std::vector<double> w;
+};
+template <typename F>
+Plan make_plan(int32_t n, int32_t m, F terms) {
+  Plan P;
+  P.rp.assign(n + 1, 0);
+  std::vector<int32_t> ci[kMaxChunks], cnt[kMaxChunks], id[kMaxChunks];
+  std::vector<double> w[kMaxChunks];
+  parallel_rows(n, [&](int32_t lo, int32_t hi, int k) {
+    std::vector<int32_t> mark(m, -1), num(m, 0), cols;
+    for (int32_t i = lo; i < hi; ++i) {
+      cols.clear();
+      int32_t total = 0;
+      terms(i, [&](int32_t j, int32_t, double) {
+        if (mark[j] != i) { mark[j] = i; num[j] = 0; cols.push_back(j); }
+        ++num[j];
+        ++total;
+      });
+      std::sort(cols.begin(), cols.end());
+      int32_t at = (int32_t)id[k].size();
+      id[k].resize(at + total);
+      w[k].resize(at + total);
+      for (int32_t j : cols) {  // num[j]: the next place of column j's terms
+        const int32_t c = num[j];
+        ci[k].push_back(j);
+        cnt[k].push_back(c);
+        num[j] = at;
+        at += c;
+      }
+      terms(i, [&](int32_t j, int32_t q, double x) {
+        id[k][num[j]] = q;
+        w[k][num[j]++] = x;
+      });
+      P.rp[i + 1] = (int32_t)cols.size();
+    }
+  });
+  for (int32_t i = 0; i < n; ++i) P.rp[i + 1] += P.rp[i];
+  P.off.assign(1, 0);
+  P.off.reserve(P.rp[n] + 1);
+  for (int k = 0; k < kMaxChunks; ++k) {
+    P.ci.insert(P.ci.end(), ci[k].begin(), ci[k].end());
+    P.id.insert(P.id.end(), id[k].begin(), id[k].end());
+    P.w.insert(P.w.end(), w[k].begin(), w[k].end());
+    for (int32_t c : cnt[k]) P.off.push_back(P.off.back() + c);
+  }
+  return P;
+}
+
+HCsr multiply(const HCsr& A, const HCsr& B) {
+  return row_sums(A.n, B.m, [&](int32_t i, auto add) {
     for (int32_t q = A.rp[i]; q < A.rp[i + 1]; ++q) {
       const int32_t k = A.ci[q];
       const double a = A.v[q];
-      for (int32_t t = B.rp[k]; t < B.rp[k + 1]; ++t) {
-        const int32_t j = B.ci[t];
-        if (mark[j] != i) { mark[j] = i; acc[j] = 0.0; cols.push_back(j); }
-        acc[j] += a * B.v[t];
-      }
+      for (int32_t t = B.rp[k]; t < B.rp[k + 1]; ++t) add(B.ci[t], a * B.v[t]);
     }
-    std::sort(cols.begin(), cols.end());
-    for (int32_t j : cols) { C.ci.push_back(j); C.v.push_back(acc[j]); }
-    C.rp[i + 1] = (int32_t)C.ci.size();
-  }
-  return C;
+  });
 }
 
 std::vector<double> diagonal(const HCsr& A) {
@@ -97,44 +208,60 @@ std::vector<double> diagonal(const HCsr& A) {
   return d;
 }
 
-// Spectral radius of D^-1 A: power iteration from a fixed non-constant
-// start, times a safety factor, capped by Gershgorin's bound.
-double spectral_radius(const HCsr& A, const std::vector<double>& d) {
-  double gersh = 0.0;
-  for (int32_t i = 0; i < A.n; ++i) {
-    double s = 0.0;
-    for (int32_t q = A.rp[i]; q < A.rp[i + 1]; ++q) s += std::fabs(A.v[q]);
-    gersh = std::max(gersh, s / d[i]);
-  }
+// A bound of the eigenvalues of D^-1 A for the dampings: twelve power
+// iterations times 1.15, at most Gershgorin's bound.  (kDamp over it stays
+// below 2 / lambda_max while the iterations reach 0.73 lambda_max.)
+double eigen_bound(const HCsr& A, const std::vector<double>& d) {
   std::vector<double> x(A.n), y(A.n);
+  double gersh[kMaxChunks] = {}, sum[kMaxChunks] = {};
   for (int32_t i = 0; i < A.n; ++i) x[i] = 1.0 + (double)((i * 7919) % 101) / 101.0;
-  double lam = 0.0;
-  for (int it = 0; it < 60; ++it) {
-    double nx = 0.0;
-    for (int32_t i = 0; i < A.n; ++i) {
-      double s = 0.0;
-      for (int32_t q = A.rp[i]; q < A.rp[i + 1]; ++q) s += A.v[q] * x[A.ci[q]];
-      y[i] = s / d[i];
-      nx += y[i] * y[i];
-    }
-    nx = std::sqrt(nx);
-    if (!(nx > 0.0)) break;
-    double xn = 0.0;
-    for (int32_t i = 0; i < A.n; ++i) xn += x[i] * x[i];
-    lam = nx / std::sqrt(xn);
-    for (int32_t i = 0; i < A.n; ++i) x[i] = y[i] / nx;
+  double lam = 0.0, nx = 1.0;
+  for (int it = 0; it < 12; ++it) {
+    parallel_rows(A.n, [&](int32_t lo, int32_t hi, int k) {
+      double s2 = 0.0, g = 0.0;
+      for (int32_t i = lo; i < hi; ++i) {
+        double s = 0.0, a = 0.0;
+        for (int32_t q = A.rp[i]; q < A.rp[i + 1]; ++q) {
+          s += A.v[q] * x[A.ci[q]];
+          a += std::fabs(A.v[q]);
+        }
+        y[i] = s / (d[i] * nx);
+        s2 += y[i] * y[i];
+        g = std::max(g, a / d[i]);
+      }
+      sum[k] = s2;
+      gersh[k] = g;
+    });
+    double t = 0.0;
+    for (double s : sum) t += s;
+    if (!(t > 0.0)) break;
+    nx = std::sqrt(t);  // (x = y / nx formed by the next product)
+    lam = it > 0 ? nx : 0.0;
+    std::swap(x, y);
   }
-  return std::min(gersh, 1.1 * lam > 0.0 ? 1.1 * lam : gersh);
+  const double g = *std::max_element(gersh, gersh + kMaxChunks);
+  return lam > 0.0 ? std::min(g, 1.15 * lam) : g;
 }
 
 // Aggregates of strongly connected unknowns: seeds whose strong
 // neighbourhood is free take it whole; leftovers join the aggregate they
 // are most strongly connected to; what remains forms new aggregates.
-std::vector<int32_t> aggregate(const HCsr& A, const std::vector<double>& d, double theta, int32_t* n_agg) {
+// A connection is strong when -a_ij >= theta sqrt(m_i m_j), m_i the largest
+// -a_ij of row i: relative to the row's strongest connection, so that on the
+// channel's flat cells (couplings across the cell 40 times those along it)
+// the coarsening follows the strong direction, and on isotropic cells takes
+// all neighbours.  (|a_ij| >= 0.08 sqrt(a_ii a_jj) also took the jittered cells'
+// middling couplings, and point smoothing then fails along the weak
+// direction: 50 iterations to 1e-12 on the 100 x 200 channel against 20.)
+std::vector<int32_t> aggregate(const HCsr& A, double theta, int32_t* n_agg) {
   const int32_t n = A.n;
+  std::vector<double> m(n, 0.0);
+  for (int32_t i = 0; i < n; ++i)
+    for (int32_t q = A.rp[i]; q < A.rp[i + 1]; ++q)
+      if (A.ci[q] != i) m[i] = std::max(m[i], -A.v[q]);
   auto strong = [&](int32_t i, int32_t q) {
     const int32_t j = A.ci[q];
-    return j != i && std::fabs(A.v[q]) >= theta * std::sqrt(std::fabs(d[i] * d[j]));
+    return j != i && A.v[q] < 0.0 && A.v[q] * A.v[q] >= theta * theta * m[i] * m[j];
   };
   std::vector<int32_t> agg(n, -1);
   int32_t na = 0;
@@ -196,83 +323,77 @@ void amg_free(Amg& G) {
   G = Amg();
 }
 
+// Damping of the Jacobi smoother over the bound of the largest eigenvalue of
+// D^-1 A (below 2 / bound: the V-cycle stays positive definite).  5/3 needs
+// about a tenth fewer iterations than the 4/3 of the prolongation's
+// smoothing on the channel and obstacle meshes.
+constexpr double kDamp = 5.0 / 3.0;
+
 // The smoothed-aggregation hierarchy of A0 down to at most kCoarse
-// unknowns: the level matrices As, prolongations Ps, Q = (I - W A) P and
-// the smoother weights W of every level, and the coarsest matrix.
-static pdf_status build_levels(HCsr A, int32_t kCoarse, std::vector<HCsr>& As, std::vector<HCsr>& Ps,
+// unknowns: the level matrices As, prolongations Ps and the coarsest matrix;
+// with_q: also Q = (I - W A) P and the smoother weights W of every level.
+static pdf_status build_levels(HCsr A, int32_t kCoarse, bool with_q, std::vector<HCsr>& As, std::vector<HCsr>& Ps,
                                std::vector<HCsr>& Qs, std::vector<std::vector<double>>& Ws, HCsr& Afinal) {
   constexpr int32_t kMaxLevels = 12;
-  double theta = 0.08;
+  double theta = 0.5;  // falls by 0.7 a level: the coarse matrices are denser and more isotropic
   while (A.n > kCoarse && (int32_t)As.size() < kMaxLevels) {
     const std::vector<double> d = diagonal(A);
     for (double x : d)
       if (!(x > 0.0)) return fail(PDF_EINVAL, "amg: non-positive diagonal");
     int32_t na = 0;
-    const std::vector<int32_t> agg = aggregate(A, d, theta, &na);
+    std::vector<int32_t> agg = aggregate(A, theta, &na);
+    // hardly any coarsening (few mutually strong connections): weaker ones count too
+    for (double t = 0.5 * theta; na > 0.7 * A.n && t > 1e-3; t *= 0.5) agg = aggregate(A, t, &na);
     if (na >= A.n || na < 1) break;
-    const double rho = spectral_radius(A, d);
-    const double wp = 4.0 / (3.0 * rho);
+    const double rho = eigen_bound(A, d);
     // P = (I - wp D^-1 A) P_tent
-    HCsr P;
-    P.n = A.n;
-    P.m = na;
-    P.rp.assign(A.n + 1, 0);
-    {
-      std::vector<int32_t> mark(na, -1), cols;
-      std::vector<double> acc(na, 0.0);
-      for (int32_t i = 0; i < A.n; ++i) {
-        cols.clear();
-        auto add = [&](int32_t c, double x) {
-          if (mark[c] != i) { mark[c] = i; acc[c] = 0.0; cols.push_back(c); }
-          acc[c] += x;
-        };
-        add(agg[i], 1.0);
-        for (int32_t q = A.rp[i]; q < A.rp[i + 1]; ++q) add(agg[A.ci[q]], -wp * A.v[q] / d[i]);
-        std::sort(cols.begin(), cols.end());
-        for (int32_t c : cols) { P.ci.push_back(c); P.v.push_back(acc[c]); }
-        P.rp[i + 1] = (int32_t)P.ci.size();
-      }
-    }
+    const double wp = 4.0 / (3.0 * rho);
+    const HCsr P = row_sums(A.n, na, [&](int32_t i, auto add) {
+      add(agg[i], 1.0);
+      for (int32_t q = A.rp[i]; q < A.rp[i + 1]; ++q) add(agg[A.ci[q]], -wp * A.v[q] / d[i]);
+    });
     const HCsr AP = multiply(A, P);
     HCsr Ac = multiply(transpose(P), AP);
-    // smoother W = ws D^-1 and Q = P - W A P
-    const double ws = 4.0 / (3.0 * rho);
-    std::vector<double> W(A.n);
-    for (int32_t i = 0; i < A.n; ++i) W[i] = ws / d[i];
-    HCsr Q;
-    Q.n = A.n;
-    Q.m = na;
-    Q.rp.assign(A.n + 1, 0);
-    {
-      std::vector<int32_t> mark(na, -1), cols;
-      std::vector<double> acc(na, 0.0);
-      for (int32_t i = 0; i < A.n; ++i) {
-        cols.clear();
-        auto add = [&](int32_t c, double x) {
-          if (mark[c] != i) { mark[c] = i; acc[c] = 0.0; cols.push_back(c); }
-          acc[c] += x;
-        };
+    if (with_q) {  // smoother W = ws D^-1 and Q = P - W A P
+      const double ws = kDamp / rho;
+      std::vector<double> W(A.n);
+      for (int32_t i = 0; i < A.n; ++i) W[i] = ws / d[i];
+      Qs.push_back(row_sums(A.n, na, [&](int32_t i, auto add) {
         for (int32_t q = P.rp[i]; q < P.rp[i + 1]; ++q) add(P.ci[q], P.v[q]);
         for (int32_t q = AP.rp[i]; q < AP.rp[i + 1]; ++q) add(AP.ci[q], -W[i] * AP.v[q]);
-        std::sort(cols.begin(), cols.end());
-        for (int32_t c : cols) { Q.ci.push_back(c); Q.v.push_back(acc[c]); }
-        Q.rp[i + 1] = (int32_t)Q.ci.size();
-      }
+      }));
+      Ws.push_back(std::move(W));
     }
-    As.push_back(A);
+    As.push_back(std::move(A));
     Ps.push_back(P);
-    Qs.push_back(Q);
-    Ws.push_back(W);
     A = std::move(Ac);
-    theta *= 0.5;
+    theta *= 0.7;
   }
   Afinal = std::move(A);
   return PDF_OK;
 }
 
+// Pressure systems of at most this many unknowns are solved by one cluster.
+constexpr int32_t kAmgWholeMax = 4096;
+
+static pdf_status amg_setup_host(int32_t n, const std::vector<int32_t>& rp, const std::vector<int32_t>& ci,
+                                 const std::vector<double>& v, bool singular, Amg& G);
+
 pdf_status amg_setup(int32_t n, const std::vector<int32_t>& rp, const std::vector<int32_t>& ci,
                      const std::vector<double>& v, bool singular, Amg& G) {
-  constexpr int32_t kCoarse = 256;
+  try {
+    return amg_setup_host(n, rp, ci, v, singular, G);
+  } catch (const std::bad_alloc&) {
+    amg_free(G);
+    return fail(PDF_ENOMEM, "amg: host allocation");
+  }
+}
+
+static pdf_status amg_setup_host(int32_t n, const std::vector<int32_t>& rp, const std::vector<int32_t>& ci,
+                     const std::vector<double>& v, bool singular, Amg& G) {
+  // (the cluster form takes the dense product in every CTA: at 256 unknowns its
+  // FP64 additions took 18 us per cycle)
+  const int32_t kCoarse = n <= kAmgWholeMax ? 64 : 256;
   HCsr A0;
   A0.n = A0.m = n;
   A0.rp = rp;
@@ -281,7 +402,7 @@ pdf_status amg_setup(int32_t n, const std::vector<int32_t>& rp, const std::vecto
   std::vector<HCsr> As, Ps, Qs;
   std::vector<std::vector<double>> Ws;
   HCsr A;
-  pdf_status bs = build_levels(A0, kCoarse, As, Ps, Qs, Ws, A);
+  pdf_status bs = build_levels(std::move(A0), kCoarse, true, As, Ps, Qs, Ws, A);
   if (bs != PDF_OK) return bs;
   // coarsest: regularised dense inverse (Gauss-Jordan with partial pivoting)
   const int32_t nc = A.n;
@@ -480,6 +601,51 @@ __global__ void __launch_bounds__(256) k_amg_up_g(int32_t n, const int32_t* __re
   if (i < n && g == 0) z[i] = x[i] + w[i] * (b[i] - ax) + qe;
 }
 
+// The levels, level 0's right-hand side r.
+static Cycle<double, 1> amg_cycle(const Amg& G, const double* r, int first, int ctas) {
+  Cycle<double, 1> C;
+  C.L = (int)G.lv.size();
+  C.first = first;
+  C.nc = G.nc;
+  C.cinv = G.cinv;
+  for (int l = 0; l < C.L; ++l) {
+    const AmgLevel& V = G.lv[l];
+    CyLevel<double, 1>& D = C.lv[l];
+    D.n = V.n; D.nc = V.nc; D.nnz_a = V.nnz_a; D.nnz_q = V.nnz_q;
+    D.a_rp = V.a_rp; D.a_ci = V.a_ci; D.q_rp = V.q_rp; D.q_ci = V.q_ci; D.s_rp = V.s_rp; D.s_ci = V.s_ci;
+    D.a[0] = V.a_v; D.q[0] = V.q_v; D.s[0] = V.s_v; D.w[0] = V.w;
+    D.b = l == 0 ? const_cast<double*>(r) : V.b;
+    D.x = V.x;
+    D.z = V.z;
+  }
+  cy_plan(C, ctas);
+  return C;
+}
+
+// The line between the two forms: one cluster against kernels per sweep, whole
+// projection calls of 20 particles per element: 748 against 960 us at 760
+// unknowns, 1,020 against 1,038 at 3,520, 1,326 against 1,170 at 6,930 (one
+// component on eight SMs is FP64-bound there).  For the same reason the large
+// form keeps a kernel per sweep on every level: a cluster for the levels
+// below 3,000 unknowns made it 4 % slower.
+bool amg_whole(const Amg& G, int32_t n) { return n <= kAmgWholeMax || G.lv.empty(); }
+
+pdf_status amg_solve(const Amg& G, const AmgSystem& A, int32_t it_end, cudaStream_t st) {
+  const int ctas = cy_ctas(A.n);
+  CySys<1> S;
+  S.n = A.n;
+  S.rp = A.rp; S.ci = A.ci; S.wall = nullptr;
+  S.a[0] = A.val;
+  S.x = A.x; S.r = A.r; S.p = A.p; S.q = A.q;
+  S.rr = A.rr; S.rz = A.rz; S.tol2 = A.tol2;
+  S.iters = A.iters; S.state = A.done;
+  S.on = 0; S.off = 1;
+  const Cycle<double, 1> C = amg_cycle(G, nullptr, 0, ctas);
+  cudaError_t e = cudaSuccess;
+  PDF_KERNEL("k_press_pcg", st, e = (cy_launch_pcg<double, 1>(1, ctas, st, S, C, it_end)));
+  return e == cudaSuccess ? PDF_OK : cuda_fail(e, "k_press_pcg");
+}
+
 pdf_status amg_apply(const Amg& G, const double* r, double* z, double* part, int32_t* counter, double* rz,
                      double* rz_old, const int32_t* done, cudaStream_t st) {
   const int32_t L = (int32_t)G.lv.size();
@@ -491,10 +657,6 @@ pdf_status amg_apply(const Amg& G, const double* r, double* z, double* part, int
     const int32_t nbx = (V.n + 255) / 256, nbc = (int32_t)(((int64_t)V.nc * kG + 255) / 256);
     PDF_KERNEL("k_amg_down", st, k_amg_down<<<nbx + nbc, 256, 0, st>>>(V.n, V.nc, nbx, V.w, V.s_rp, V.s_ci, V.s_v, b,
                                                                         V.x, bc, done));
-  }
-  if (L == 0) {
-    PDF_KERNEL("k_amg_coarse", st, k_amg_coarse<<<(G.nc + 7) / 8, 256, 0, st>>>(G.nc, G.cinv, r, z, done));
-    return PDF_OK;
   }
   PDF_KERNEL("k_amg_coarse", st, k_amg_coarse<<<(G.nc + 7) / 8, 256, 0, st>>>(G.nc, G.cinv, G.cb, G.cz, done));
   for (int32_t l = L - 1; l >= 0; --l) {
@@ -760,13 +922,26 @@ void relax_amg_free(RelaxAmg& G) {
   }
   cudaFree(G.c_rp); cudaFree(G.c_ci);
   for (int v = 0; v < kRxVar; ++v) cudaFree(G.c_v[v]);
-  cudaFree(G.cmat); cudaFree(G.cinv); cudaFree(G.cb); cudaFree(G.cz); cudaFree(G.omega); cudaFree(G.gpart);
+  cudaFree(G.cmat); cudaFree(G.cinv); cudaFree(G.r32); cudaFree(G.omega); cudaFree(G.gpart);
   cudaFree(G.upart);
   G = RelaxAmg();
 }
 
+static pdf_status relax_amg_setup_host(int32_t n, const std::vector<int32_t>& rp, const std::vector<int32_t>& ci,
+                                       const std::vector<double>& kv, RelaxAmg& G);
+
 pdf_status relax_amg_setup(int32_t n, const std::vector<int32_t>& rp, const std::vector<int32_t>& ci,
                            const std::vector<double>& kv, RelaxAmg& G) {
+  try {
+    return relax_amg_setup_host(n, rp, ci, kv, G);
+  } catch (const std::bad_alloc&) {
+    relax_amg_free(G);
+    return fail(PDF_ENOMEM, "relax multigrid: host allocation");
+  }
+}
+
+static pdf_status relax_amg_setup_host(int32_t n, const std::vector<int32_t>& rp, const std::vector<int32_t>& ci,
+                                       const std::vector<double>& kv, RelaxAmg& G) {
   HCsr K;
   K.n = K.m = n;
   K.rp = rp;
@@ -775,7 +950,7 @@ pdf_status relax_amg_setup(int32_t n, const std::vector<int32_t>& rp, const std:
   std::vector<HCsr> As, Ps, Qs;
   std::vector<std::vector<double>> Ws;
   HCsr Afinal;
-  pdf_status s = build_levels(K, 64, As, Ps, Qs, Ws, Afinal);
+  pdf_status s = build_levels(std::move(K), 64, false, As, Ps, Qs, Ws, Afinal);
   if (s != PDF_OK) return s;
   if ((int)As.size() > kRxMaxLv) return fail(PDF_EINVAL, "relax multigrid: too many levels");
   relax_amg_free(G);
@@ -798,36 +973,24 @@ pdf_status relax_amg_setup(int32_t n, const std::vector<int32_t>& rp, const std:
     for (int32_t i = 0; i < na; ++i)
       if (dpos[i] < 0) return fail(PDF_EINVAL, "relax multigrid: missing diagonal");
     // plan of A P: per row, the (A entry, P value) pairs of each column
-    std::vector<int32_t> q_rp(na + 1, 0), q_ci, ap_off(1, 0), ap_qa, q_row;
-    std::vector<double> ap_pv, q_pin;
-    {
-      std::vector<int32_t> mark(P.m, -1), cols;
-      std::vector<std::vector<std::pair<int32_t, double>>> lists(P.m);
-      for (int32_t i = 0; i < na; ++i) {
-        cols.clear();
-        for (int32_t q = a_rp[i]; q < a_rp[i + 1]; ++q) {
-          const int32_t j = a_ci[q];
-          for (int32_t t = P.rp[j]; t < P.rp[j + 1]; ++t) {
-            const int32_t J = P.ci[t];
-            if (mark[J] != i) { mark[J] = i; lists[J].clear(); cols.push_back(J); }
-            lists[J].push_back({q, P.v[t]});
-          }
-        }
-        std::sort(cols.begin(), cols.end());
-        for (int32_t J : cols) {
-          q_ci.push_back(J);
-          q_row.push_back(i);
-          for (auto& pr : lists[J]) { ap_qa.push_back(pr.first); ap_pv.push_back(pr.second); }
-          ap_off.push_back((int32_t)ap_qa.size());
-          double pin = 0.0;
-          for (int32_t t = P.rp[i]; t < P.rp[i + 1]; ++t)
-            if (P.ci[t] == J) pin = P.v[t];
-          q_pin.push_back(pin);
-        }
-        q_rp[i + 1] = (int32_t)q_ci.size();
+    const Plan ap = make_plan(na, P.m, [&](int32_t i, auto add) {
+      for (int32_t q = a_rp[i]; q < a_rp[i + 1]; ++q) {
+        const int32_t j = a_ci[q];
+        for (int32_t t = P.rp[j]; t < P.rp[j + 1]; ++t) add(P.ci[t], q, P.v[t]);
+      }
+    });
+    const std::vector<int32_t>&q_rp = ap.rp, &q_ci = ap.ci;
+    const int64_t nap = (int64_t)q_ci.size();
+    std::vector<int32_t> q_row(nap);
+    std::vector<double> q_pin(nap, 0.0);  // P at each position (both rows ascending)
+    for (int32_t i = 0; i < na; ++i) {
+      int32_t t = P.rp[i];
+      for (int32_t k = q_rp[i]; k < q_rp[i + 1]; ++k) {
+        q_row[k] = i;
+        while (t < P.rp[i + 1] && P.ci[t] < q_ci[k]) ++t;
+        if (t < P.rp[i + 1] && P.ci[t] == q_ci[k]) q_pin[k] = P.v[t];
       }
     }
-    const int64_t nap = (int64_t)q_ci.size();
     L.nnz_ap = nap;
     // S = Q^T with the permutation of the entries
     std::vector<int32_t> s_rp(P.m + 1, 0), s_ci(nap), s_perm(nap);
@@ -843,49 +1006,20 @@ pdf_status relax_amg_setup(int32_t n, const std::vector<int32_t>& rp, const std:
         }
     }
     // plan of the next matrix, P^T (A P): coarse entry (I, J) sums P_iI (A P)_iJ
-    std::vector<int32_t> n_rp(P.m + 1, 0), n_ci, c_off(1, 0), c_tap;
-    std::vector<double> c_pv;
-    {
-      // transpose of P for the rows of the coarse matrix
-      std::vector<int32_t> pt_rp(P.m + 1, 0), pt_i(P.ci.size());
-      std::vector<double> pt_v(P.ci.size());
-      for (int32_t c : P.ci) pt_rp[c + 1]++;
-      for (int32_t I = 0; I < P.m; ++I) pt_rp[I + 1] += pt_rp[I];
-      std::vector<int32_t> fill(pt_rp.begin(), pt_rp.end() - 1);
-      for (int32_t i = 0; i < na; ++i)
-        for (int32_t t = P.rp[i]; t < P.rp[i + 1]; ++t) {
-          const int32_t d = fill[P.ci[t]]++;
-          pt_i[d] = i;
-          pt_v[d] = P.v[t];
-        }
-      std::vector<int32_t> mark(P.m, -1), cols;
-      std::vector<std::vector<std::pair<int32_t, double>>> lists(P.m);
-      for (int32_t I = 0; I < P.m; ++I) {
-        cols.clear();
-        for (int32_t k = pt_rp[I]; k < pt_rp[I + 1]; ++k) {
-          const int32_t i = pt_i[k];
-          for (int32_t t = q_rp[i]; t < q_rp[i + 1]; ++t) {
-            const int32_t J = q_ci[t];
-            if (mark[J] != I) { mark[J] = I; lists[J].clear(); cols.push_back(J); }
-            lists[J].push_back({t, pt_v[k]});
-          }
-        }
-        std::sort(cols.begin(), cols.end());
-        for (int32_t J : cols) {
-          n_ci.push_back(J);
-          for (auto& pr : lists[J]) { c_tap.push_back(pr.first); c_pv.push_back(pr.second); }
-          c_off.push_back((int32_t)c_tap.size());
-        }
-        n_rp[I + 1] = (int32_t)n_ci.size();
+    const HCsr Pt = transpose(P);
+    Plan nx = make_plan(P.m, P.m, [&](int32_t I, auto add) {
+      for (int32_t k = Pt.rp[I]; k < Pt.rp[I + 1]; ++k) {
+        const int32_t i = Pt.ci[k];
+        for (int32_t t = q_rp[i]; t < q_rp[i + 1]; ++t) add(q_ci[t], t, Pt.v[k]);
       }
-    }
+    });
     if ((s = up_vec(&L.a_rp, a_rp)) != PDF_OK || (s = up_vec(&L.a_ci, a_ci)) != PDF_OK ||
         (s = up_vec(&L.a_dpos, dpos)) != PDF_OK || (s = up_vec(&L.q_rp, q_rp)) != PDF_OK ||
         (s = up_vec(&L.q_ci, q_ci)) != PDF_OK || (s = up_vec(&L.s_rp, s_rp)) != PDF_OK ||
         (s = up_vec(&L.s_ci, s_ci)) != PDF_OK || (s = up_vec(&L.s_perm, s_perm)) != PDF_OK ||
-        (s = up_vec(&L.ap_off, ap_off)) != PDF_OK || (s = up_vec(&L.ap_qa, ap_qa)) != PDF_OK ||
-        (s = up_vec(&L.ap_pv, ap_pv)) != PDF_OK || (s = up_vec(&L.c_off, c_off)) != PDF_OK ||
-        (s = up_vec(&L.c_tap, c_tap)) != PDF_OK || (s = up_vec(&L.c_pv, c_pv)) != PDF_OK ||
+        (s = up_vec(&L.ap_off, ap.off)) != PDF_OK || (s = up_vec(&L.ap_qa, ap.id)) != PDF_OK ||
+        (s = up_vec(&L.ap_pv, ap.w)) != PDF_OK || (s = up_vec(&L.c_off, nx.off)) != PDF_OK ||
+        (s = up_vec(&L.c_tap, nx.id)) != PDF_OK || (s = up_vec(&L.c_pv, nx.w)) != PDF_OK ||
         (s = up_vec(&L.q_pin, q_pin)) != PDF_OK || (s = up_vec(&L.q_row, q_row)) != PDF_OK)
       break;
     for (int v = 0; v < kRxVar && s == PDF_OK; ++v)
@@ -899,11 +1033,13 @@ pdf_status relax_amg_setup(int32_t n, const std::vector<int32_t>& rp, const std:
     if ((s = zeros(&L.x, 9 * (int64_t)na)) != PDF_OK) break;
     if (l > 0 && ((s = zeros(&L.b, 9 * (int64_t)na)) != PDF_OK || (s = zeros(&L.z, 9 * (int64_t)na)) != PDF_OK))
       break;
-    a_rp = n_rp;
-    a_ci = n_ci;
+    a_rp = std::move(nx.rp);
+    a_ci = std::move(nx.ci);
     na = P.m;
   }
   if (s == PDF_OK && na > 64) s = fail(PDF_EINVAL, "relax multigrid: coarsest level above 64 unknowns");
+  if (s == PDF_OK && G.lv.size() < 2 && !relax_mg_whole(n))
+    s = fail(PDF_EINVAL, "relax multigrid: fewer than two levels");  // (the large form needs two)
   if (s == PDF_OK) {
     G.nc = na;
     G.nnz_c = (int64_t)a_ci.size();
@@ -912,8 +1048,7 @@ pdf_status relax_amg_setup(int32_t n, const std::vector<int32_t>& rp, const std:
     for (int v = 0; v < kRxVar && s == PDF_OK; ++v) s = zeros(&G.c_v[v], G.nnz_c);
     if (s == PDF_OK) s = zeros(&G.cmat, (int64_t)kRxVar * na * 2 * na);
     if (s == PDF_OK) s = zeros(&G.cinv, (int64_t)kRxVar * na * na);
-    if (s == PDF_OK) s = zeros(&G.cb, 9 * (int64_t)na);
-    if (s == PDF_OK) s = zeros(&G.cz, 9 * (int64_t)na);
+    if (s == PDF_OK) s = zeros(&G.r32, 9 * (int64_t)n);
     if (s == PDF_OK) s = zeros(&G.omega, kRxVar * kRxMaxLv);
     G.gblocks = (int32_t)std::min<int64_t>(1024, ((int64_t)n + 255) / 256);
     if (s == PDF_OK) s = zeros(&G.gpart, (int64_t)kRxVar * G.gblocks);
@@ -980,7 +1115,7 @@ __global__ void k_rx_omega(const double* __restrict__ part, int32_t nb, int leve
   if (v >= kRxVar) return;
   double m = 0.0;
   for (int32_t b = 0; b < nb; ++b) m = fmax(m, part[(int64_t)v * nb + b]);
-  omega[v * kRxMaxLv + level] = m > 0.0 ? 4.0 / (3.0 * m) : 0.0;
+  omega[v * kRxMaxLv + level] = m > 0.0 ? kDamp / m : 0.0;
 }
 
 // The smoother weights W = omega / a_ii (FP64 and FP32) and the FP32 copy
@@ -1114,225 +1249,6 @@ pdf_status relax_amg_update(RelaxAmg& G, cudaStream_t st) {
     R.an[v] = G.c_v[v];
   }
   PDF_KERNEL("k_rx_coarse_inv", st, k_rx_coarse_inv<<<kRxVar, 256, 0, st>>>(G.nc, G.c_rp, G.c_ci, R, G.cmat, G.cinv));
-  return PDF_OK;
-}
-
-__device__ __forceinline__ int rx_variant(int c) { return c == 0 ? 0 : (c == 4 ? 1 : (c == 8 ? 2 : 3)); }
-
-struct RxLevelDev {
-  int32_t n, nc;
-  const int32_t *a_rp, *a_ci, *q_rp, *q_ci, *s_rp, *s_ci;
-  const float *a_f[kRxVar], *q_f[kRxVar], *s_f[kRxVar], *w_f[kRxVar];
-};
-
-template <int G>
-__device__ __forceinline__ float group_sum_f(float v) {
-#pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// x_c = W b_c on the level's rows; b_{c, next} = S b_c on the coarse rows
-// (G lanes per row: 32 where the rows of S are long), component c =
-// blockIdx.y.  FP32 arithmetic; TB the type of b (FP64 at the finest level).
-template <typename TB, int G>
-__global__ void __launch_bounds__(256) k_rx_down(RxLevelDev V, int32_t nbx, const TB* __restrict__ b,
-                                                 float* __restrict__ x, float* __restrict__ bc,
-                                                 const int32_t* __restrict__ active, const int32_t* __restrict__ done) {
-  const int c = blockIdx.y;
-  if (*done || !active[c]) return;
-  const int v = rx_variant(c);
-  const TB* bb = b + (int64_t)c * V.n;
-  if ((int32_t)blockIdx.x < nbx) {
-    const int32_t i = blockIdx.x * 256 + threadIdx.x;
-    if (i < V.n) x[(int64_t)c * V.n + i] = V.w_f[v][i] * (float)bb[i];
-  } else {
-    const int32_t J = ((blockIdx.x - nbx) * 256 + threadIdx.x) / G, g = threadIdx.x % G;
-    float s = 0.0f;
-    if (J < V.nc) {
-      const float* sv = V.s_f[v];
-      for (int32_t q = V.s_rp[J] + g; q < V.s_rp[J + 1]; q += G) s += sv[q] * (float)bb[V.s_ci[q]];
-    }
-    s = group_sum_f<G>(s);
-    if (J < V.nc && g == 0) bc[(int64_t)c * V.nc + J] = s;
-  }
-}
-
-template <typename TB, typename TZ>
-__global__ void __launch_bounds__(256) k_rx_coarse(int32_t nc, const float* __restrict__ cinv,
-                                                   const TB* __restrict__ b, TZ* __restrict__ z,
-                                                   const int32_t* __restrict__ active,
-                                                   const int32_t* __restrict__ done) {
-  const int c = blockIdx.y;
-  if (*done || !active[c]) return;
-  const int v = rx_variant(c);
-  const int32_t row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= nc) return;
-  const float* Ci = cinv + (int64_t)v * nc * nc + (int64_t)row * nc;
-  const TB* bb = b + (int64_t)c * nc;
-  float s = 0.0f;
-  for (int32_t k = lane; k < nc; k += 32) s += Ci[k] * (float)bb[k];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) z[(int64_t)c * nc + row] = (TZ)s;
-}
-
-// z_c = x_c + W (b_c - A x_c) + Q e_c on a coarse level, kG lanes per row.
-__global__ void __launch_bounds__(256) k_rx_up(RxLevelDev V, const float* __restrict__ b, const float* __restrict__ x,
-                                               const float* __restrict__ ec, float* __restrict__ z,
-                                               const int32_t* __restrict__ active, const int32_t* __restrict__ done) {
-  const int c = blockIdx.y;
-  if (*done || !active[c]) return;
-  const int v = rx_variant(c);
-  const int32_t i = (blockIdx.x * 256 + threadIdx.x) / kG, g = threadIdx.x % kG;
-  const float* xx = x + (int64_t)c * V.n;
-  const float* ee = ec + (int64_t)c * V.nc;
-  float ax = 0.0f, qe = 0.0f;
-  if (i < V.n) {
-    const float *av = V.a_f[v], *qv = V.q_f[v];
-    for (int32_t q = V.a_rp[i] + g; q < V.a_rp[i + 1]; q += kG) ax += av[q] * xx[V.a_ci[q]];
-    for (int32_t q = V.q_rp[i] + g; q < V.q_rp[i + 1]; q += kG) qe += qv[q] * ee[V.q_ci[q]];
-  }
-  ax = group_sum_f<kG>(ax);
-  qe = group_sum_f<kG>(qe);
-  if (i < V.n && g == 0) {
-    const int64_t o = (int64_t)c * V.n + i;
-    z[o] = xx[i] + V.w_f[v][i] * (b[o] - ax) + qe;
-  }
-}
-
-__device__ __forceinline__ bool rx_fixed(int c, uint8_t w) { return w == 2 || (w == 1 && c != 0 && c != 4 && c != 8); }
-
-// The finest up-sweep (one thread per row) with the application's end
-// (RxDot): z = 0 on fixed unknowns, r . z and beta.
-__device__ void rx_dot_finish(int c, double rz, double* __restrict__ part, const RxDot& D) {
-  __shared__ double sh[8];
-  __shared__ bool last;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) rz += __shfl_xor_sync(0xffffffffu, rz, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = rz;
-  __syncthreads();
-  double* pc = part + (int64_t)c * gridDim.x;
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int k = 0; k < 8; ++k) t += sh[k];
-    pc[blockIdx.x] = t;
-    __threadfence();
-    last = atomicAdd(D.counter + c, 1) == (int32_t)gridDim.x - 1;
-    if (last) D.counter[c] = 0;
-  }
-  __syncthreads();
-  if (!last) return;
-  double t = 0.0;
-  for (int32_t k = threadIdx.x; k < (int32_t)gridDim.x; k += 256) t += __ldcg(pc + k);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = t;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double v = 0.0;
-    for (int k = 0; k < 8; ++k) v += sh[k];
-    const double old = D.rz[c];
-    D.beta[c] = D.first || old == 0.0 ? 0.0 : v / old;
-    D.rz[c] = v;
-  }
-}
-
-__global__ void __launch_bounds__(256) k_rx_up0(RxLevelDev V, const double* __restrict__ r,
-                                                const float* __restrict__ x, const float* __restrict__ ec,
-                                                double* __restrict__ z, double* __restrict__ part, RxDot D,
-                                                const int32_t* __restrict__ active,
-                                                const int32_t* __restrict__ done) {
-  const int c = blockIdx.y;
-  if (*done || !active[c]) return;
-  const int v = rx_variant(c);
-  const int32_t i = blockIdx.x * 256 + threadIdx.x;
-  double rz = 0.0;
-  if (i < V.n) {
-    const int64_t o = (int64_t)c * V.n + i;
-    double zi = 0.0;
-    if (!rx_fixed(c, D.wall[i])) {
-      const float* xx = x + (int64_t)c * V.n;
-      const float* ee = ec + (int64_t)c * V.nc;
-      const float *av = V.a_f[v], *qv = V.q_f[v];
-      float ax = 0.0f, qe = 0.0f;
-      for (int32_t q = V.a_rp[i]; q < V.a_rp[i + 1]; ++q) ax += av[q] * xx[V.a_ci[q]];
-      for (int32_t q = V.q_rp[i]; q < V.q_rp[i + 1]; ++q) qe += qv[q] * ee[V.q_ci[q]];
-      const double ri = r[o];
-      zi = (double)(xx[i] + V.w_f[v][i] * ((float)ri - ax) + qe);
-      rz = ri * zi;
-    }
-    z[o] = zi;
-  }
-  rx_dot_finish(c, rz, part, D);
-}
-
-// Without levels: z = Inv r in FP32, then the same end.
-__global__ void __launch_bounds__(256) k_rx_dot(int32_t n, const double* __restrict__ r, double* __restrict__ z,
-                                                double* __restrict__ part, RxDot D, const int32_t* __restrict__ active,
-                                                const int32_t* __restrict__ done) {
-  const int c = blockIdx.y;
-  if (*done || !active[c]) return;
-  const int32_t i = blockIdx.x * 256 + threadIdx.x;
-  double rz = 0.0;
-  if (i < n) {
-    const int64_t o = (int64_t)c * n + i;
-    if (rx_fixed(c, D.wall[i])) z[o] = 0.0;
-    else rz = r[o] * z[o];
-  }
-  rx_dot_finish(c, rz, part, D);
-}
-
-pdf_status relax_amg_apply(const RelaxAmg& G, const double* r, double* z, const int32_t* active,
-                           const int32_t* done, const RxDot& dot, cudaStream_t st) {
-  const int L = (int)G.lv.size();
-  auto dev = [&](int l) {
-    const RxLevel& V = G.lv[l];
-    RxLevelDev D;
-    D.n = V.n;
-    D.nc = V.nc;
-    D.a_rp = V.a_rp; D.a_ci = V.a_ci;
-    D.q_rp = V.q_rp; D.q_ci = V.q_ci; D.s_rp = V.s_rp; D.s_ci = V.s_ci;
-    for (int v = 0; v < kRxVar; ++v) { D.a_f[v] = V.a_f[v]; D.q_f[v] = V.q_f[v]; D.s_f[v] = V.s_f[v]; D.w_f[v] = V.w_f[v]; }
-    return D;
-  };
-  if (L == 0) {
-    PDF_KERNEL("k_rx_coarse", st, (k_rx_coarse<double, double><<<dim3((G.nc + 7) / 8, 9), 256, 0, st>>>(
-                                      G.nc, G.cinv, r, z, active, done)));
-    PDF_KERNEL("k_rx_dot", st, k_rx_dot<<<dim3((G.nc + 255) / 256, 9), 256, 0, st>>>(G.nc, r, z, G.upart, dot,
-                                                                                       active, done));
-    return PDF_OK;
-  }
-  for (int l = 0; l < L; ++l) {
-    const RxLevel& V = G.lv[l];
-    float* bc = l + 1 < L ? G.lv[l + 1].b : G.cb;
-    // a warp per coarse row where the rows of S are long
-    const bool wide = V.nnz_ap > 48 * (int64_t)V.nc;
-    const int lanes = wide ? 32 : kG;
-    const int32_t nbx = (V.n + 255) / 256, nbc = (int32_t)(((int64_t)V.nc * lanes + 255) / 256);
-    const dim3 grid(nbx + nbc, 9);
-    if (l == 0 && wide)
-      PDF_KERNEL("k_rx_down", st, (k_rx_down<double, 32><<<grid, 256, 0, st>>>(dev(l), nbx, r, V.x, bc, active, done)));
-    else if (l == 0)
-      PDF_KERNEL("k_rx_down", st, (k_rx_down<double, kG><<<grid, 256, 0, st>>>(dev(l), nbx, r, V.x, bc, active, done)));
-    else if (wide)
-      PDF_KERNEL("k_rx_down", st, (k_rx_down<float, 32><<<grid, 256, 0, st>>>(dev(l), nbx, V.b, V.x, bc, active, done)));
-    else
-      PDF_KERNEL("k_rx_down", st, (k_rx_down<float, kG><<<grid, 256, 0, st>>>(dev(l), nbx, V.b, V.x, bc, active, done)));
-  }
-  PDF_KERNEL("k_rx_coarse", st, (k_rx_coarse<float, float><<<dim3((G.nc + 7) / 8, 9), 256, 0, st>>>(
-                                    G.nc, G.cinv, G.cb, G.cz, active, done)));
-  for (int l = L - 1; l >= 0; --l) {
-    const RxLevel& V = G.lv[l];
-    const float* ec = l + 1 < L ? G.lv[l + 1].z : G.cz;
-    if (l == 0)
-      PDF_KERNEL("k_rx_up0", st, k_rx_up0<<<dim3((V.n + 255) / 256, 9), 256, 0, st>>>(dev(l), r, V.x, ec, z, G.upart,
-                                                                                       dot, active, done));
-    else
-      PDF_KERNEL("k_rx_up", st, k_rx_up<<<dim3((int32_t)(((int64_t)V.n * kG + 255) / 256), 9), 256, 0, st>>>(
-                                    dev(l), V.b, V.x, ec, V.z, active, done));
-  }
   return PDF_OK;
 }
 

@@ -32,12 +32,25 @@ struct Amg {
 pdf_status amg_setup(int32_t n, const std::vector<int32_t>& rp, const std::vector<int32_t>& ci,
                      const std::vector<double>& v, bool singular, Amg& G);
 void amg_free(Amg& G);
-// z = M^-1 r (one V-cycle).  When the hierarchy has a level, the finest
-// up-sweep also forms r . z (block partials in part, finished by the last
-// block through *counter, which it resets): *rz_old = *rz, *rz = r . z;
-// else the caller forms it.  Every kernel returns at once when *done is set.
+// z = M^-1 r (one V-cycle; a level at least).  The finest up-sweep also
+// forms r . z (block partials in part, finished by the last block through
+// *counter, which it resets): *rz_old = *rz, *rz = r . z.  Every kernel returns
+// at once when *done is set.
 pdf_status amg_apply(const Amg& G, const double* r, double* z, double* part, int32_t* counter, double* rz,
                      double* rz_old, const int32_t* done, cudaStream_t st);
+
+// The whole preconditioned conjugate-gradient solve of a system of n
+// unknowns by one cluster in one launch, up to iteration it_end (*done = 1 at
+// r.r <= *tol2 or a breakdown); amg_whole: whether a system takes this form.
+struct AmgSystem {
+  int32_t n = 0;
+  const int32_t *rp = nullptr, *ci = nullptr;
+  const double* val = nullptr;
+  double *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *rr = nullptr, *rz = nullptr, *tol2 = nullptr;
+  int32_t *iters = nullptr, *done = nullptr;
+};
+bool amg_whole(const Amg& G, int32_t n);
+pdf_status amg_solve(const Amg& G, const AmgSystem& A, int32_t it_end, cudaStream_t st);
 
 // The whole preconditioned conjugate-gradient iteration for the CSR matrix
 // (n rows; rp, ci, val) in one persistent cooperative kernel, the phases
@@ -82,7 +95,7 @@ struct RxLevel {
   double* w_v[kRxVar] = {};  // smoother weights W = omega / a_ii
   // FP32 copies for the cycle: A, Q, S and W
   float *a_f[kRxVar] = {}, *q_f[kRxVar] = {}, *s_f[kRxVar] = {}, *w_f[kRxVar] = {};
-  float *b = nullptr, *x = nullptr, *z = nullptr;                // [9][n] (b, z for l > 0)
+  float *b = nullptr, *x = nullptr, *z = nullptr;                // [9][n] (b, z for l > 0; level 0's b is r32)
 };
 
 struct RelaxAmg {
@@ -93,23 +106,30 @@ struct RelaxAmg {
   double* c_v[kRxVar] = {};
   double* cmat = nullptr;                    // [kRxVar][nc][2 nc] Gauss-Jordan work
   float* cinv = nullptr;                     // [kRxVar][nc][nc]
-  float *cb = nullptr, *cz = nullptr;        // [9][nc]
+  float* r32 = nullptr;                      // [9][n] FP32 residual, the finest level's b
   double *omega = nullptr, *gpart = nullptr; // [kRxVar][kRxMaxLv], Gershgorin partial maxima
   int32_t gblocks = 0;
   double* upart = nullptr;                   // [9][blocks of the finest up-sweep], r . z partials
 };
 
-// The end of a preconditioner application: z = 0 on the fixed unknowns
-// (wall[i] == 2 for every component; wall[i] == 1 also for the off-diagonal
-// components c != 0, 4, 8) and r . z per component, whose last block sets
-// beta[c] = (first ? 0 : r.z / rz[c]), rz[c] = r.z and returns counter[c]
-// to 0.
-struct RxDot {
+// Device scalars (9 components each) and control words of the relaxation's
+// conjugate gradients.
+enum { kRPq = 0, kRRz = 9, kRRr = 18, kRBb = 27, kRTol2 = 36, kRAlpha = 45, kRBeta = 54 };
+enum { kRDone = 0, kRIt = 1, kRMaxIt = 2, kRCntClose = 3, kRCntUp0 = 4, kRCntSpmv = 8, kRCntUpd = 17, kRActive = 26,
+       kRIters = 35 };
+
+// The nine components' systems (the matrices are the hierarchy's finest
+// ones, on the pattern rp / ci) and the iteration's vectors
+// ([9][n] each), as the caller's initialisation leaves them: x, r = b - A x,
+// scal (r.r, the thresholds), ctl (active components, max_it).  wall[i]
+// marks fixed unknowns (2 for every component; 1 for the off-diagonal
+// components c != 0, 4, 8).  part: 18 doubles per 256 unknowns.
+struct RxSystem {
+  int32_t n = 0;
+  const int32_t *rp = nullptr, *ci = nullptr;
   const uint8_t* wall = nullptr;
-  double* rz = nullptr;       // [9]
-  double* beta = nullptr;     // [9]
-  int32_t* counter = nullptr; // [9]
-  int first = 0;
+  double *x = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr, *part = nullptr, *scal = nullptr;
+  int32_t* ctl = nullptr;
 };
 
 // Plans from the hierarchy of K (n unknowns, CSR rp / ci / kv), coarsest
@@ -124,11 +144,17 @@ inline double* relax_amg_level0(RelaxAmg& G, int v) { return G.lv.empty() ? G.c_
 // inverses of the coarsest matrices of the four variants, from the finest
 // values (fixed unknowns with their diagonal only).
 pdf_status relax_amg_update(RelaxAmg& G, cudaStream_t st);
-// z = M^-1 r for the nine components ([9][n] each; component c uses
-// variant 0, 1, 2 for c = 0, 4, 8 and 3 otherwise); components with
-// active[c] = 0 and everything after *done are skipped.  The cycle runs in
-// FP32 (the level matrices and vectors), r and z are FP64.
-pdf_status relax_amg_apply(const RelaxAmg& G, const double* r, double* z, const int32_t* active,
-                           const int32_t* done, const RxDot& dot, cudaStream_t st);
+// The conjugate gradients preconditioned by one V-cycle per iteration
+// (relax_pcg.cu); component c uses variant 0, 1, 2 for c = 0, 4, 8 and 3
+// otherwise.  The cycle runs in FP32 (level matrices and vectors), the
+// rest in FP64.  relax_mg_whole: whether a system of n unknowns runs its whole
+// solve up to iteration it_end in one launch (relax_mg_solve, which leaves
+// scal[kRRr], ctl[kRIters] and ctl[kRActive], 0 for the converged components) or by relax_mg_begin (the first
+// z = M^-1 r) and chunks of relax_mg_iterations (kernels that return at once
+// when ctl[kRDone] is set).
+bool relax_mg_whole(int32_t n);
+pdf_status relax_mg_solve(const RelaxAmg& G, const RxSystem& A, int32_t it_end, cudaStream_t st);
+pdf_status relax_mg_begin(const RelaxAmg& G, const RxSystem& A, cudaStream_t st);
+pdf_status relax_mg_iterations(const RelaxAmg& G, const RxSystem& A, int k, cudaStream_t st);
 
 }  // namespace pdfgb

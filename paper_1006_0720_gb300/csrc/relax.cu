@@ -211,10 +211,6 @@ __global__ void k_cg_reduce(const double* __restrict__ part, int32_t nb, int32_t
   if (threadIdx.x == 0) out[q] = s;
 }
 
-// Device scalars (9 components each) and control words of the iteration.
-enum { kRPq = 0, kRRz = 9, kRRr = 18, kRBb = 27, kRTol2 = 36, kRAlpha = 45, kRBeta = 54 };
-enum { kRDone = 0, kRIt = 1, kRMaxIt = 2, kRCntSpmv = 8, kRCntUpd = 17, kRActive = 26, kRIters = 35 };
-
 // True in the block of component blockIdx.y that arrives last (its partial
 // written before); it resets the counter.
 __device__ __forceinline__ bool last_block_of(int32_t* counter) {
@@ -376,69 +372,6 @@ __global__ void k_rx_fill(int32_t n_rep, int64_t nnz, const int32_t* __restrict_
   }
 }
 
-// Multigrid path: p = z + beta p, q = A z + beta q (= A p) and p.q (last
-// block of a component: alpha = r.z / p.q).
-__global__ void __launch_bounds__(kRBlock) k_cg_spmv_rec(int32_t n_rep, int64_t nnz, const int32_t* __restrict__ rp,
-                                                          const int32_t* __restrict__ ci,
-                                                          const double* __restrict__ aval,
-                                                          const uint8_t* __restrict__ wall,
-                                                          const double* __restrict__ z, double* __restrict__ p,
-                                                          double* __restrict__ q, double* __restrict__ part,
-                                                          double* __restrict__ scal, int32_t* __restrict__ ctl) {
-  const int ij = blockIdx.y;
-  if (ctl[kRDone] || !ctl[kRActive + ij]) return;
-  const int32_t row = blockIdx.x * kRBlock + threadIdx.x;
-  double pq = 0.0;
-  if (row < n_rep) {
-    const double beta = scal[kRBeta + ij];
-    const int64_t o = (int64_t)ij * n_rep + row;
-    const double qn = spmv_row(row, ij, n_rep, nnz, rp, ci, aval, wall, z) + beta * q[o];
-    const double pn = z[o] + beta * p[o];
-    q[o] = qn;
-    p[o] = pn;
-    pq = qn * pn;
-  }
-  double* pp = part + (int64_t)ij * gridDim.x;
-  const double s = block_sum(pq);
-  if (threadIdx.x == 0) pp[blockIdx.x] = s;
-  if (!last_block_of(ctl + kRCntSpmv + ij)) return;
-  const double t = sum_of(pp, gridDim.x);
-  if (threadIdx.x == 0) {
-    scal[kRPq + ij] = t;
-    scal[kRAlpha + ij] = t != 0.0 ? scal[kRRz + ij] / t : 0.0;
-  }
-}
-
-// x += alpha p; r -= alpha q; r.r (last block of a component: count the
-// iteration, retire the component at r.r <= rtol^2 b.b).
-__global__ void __launch_bounds__(kRBlock) k_cg_update_mg(int32_t n_rep, double* __restrict__ scal,
-                                                           double* __restrict__ x, double* __restrict__ r,
-                                                           const double* __restrict__ p, const double* __restrict__ q,
-                                                           double* __restrict__ part, int32_t* __restrict__ ctl) {
-  const int ij = blockIdx.y;
-  if (ctl[kRDone] || !ctl[kRActive + ij]) return;
-  const int32_t row = blockIdx.x * kRBlock + threadIdx.x;
-  double rr = 0.0;
-  if (row < n_rep) {
-    const double alpha = scal[kRAlpha + ij];
-    const int64_t o = (int64_t)ij * n_rep + row;
-    x[o] += alpha * p[o];
-    const double res = r[o] - alpha * q[o];
-    r[o] = res;
-    rr = res * res;
-  }
-  double* p2 = part + (int64_t)(18 + ij) * gridDim.x;
-  const double s2 = block_sum(rr);
-  if (threadIdx.x == 0) p2[blockIdx.x] = s2;
-  if (!last_block_of(ctl + kRCntUpd + ij)) return;
-  const double rrn = sum_of(p2, gridDim.x);
-  if (threadIdx.x == 0) {
-    scal[kRRr + ij] = rrn;
-    ctl[kRIters + ij] += 1;
-    if (rrn <= scal[kRTol2 + ij]) ctl[kRActive + ij] = 0;
-  }
-}
-
 __global__ void k_cg_diag(int32_t n_rep, int64_t nnz, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                           const double* __restrict__ aval, double* __restrict__ diag) {
   const int cl = blockIdx.y;
@@ -509,7 +442,7 @@ static pdf_status relax_alloc(pdf_particles* P) {
   A((void**)&W.z, sizeof(double) * 9 * R.n_rep);
   A((void**)&W.p, sizeof(double) * 9 * R.n_rep);
   A((void**)&W.q, sizeof(double) * 9 * R.n_rep);
-  A((void**)&W.part, sizeof(double) * 3 * 9 * nb);
+  A((void**)&W.part, sizeof(double) * 3 * 9 * nb);  // (>= 18 per 256 unknowns for the multigrid path)
   A((void**)&W.scal, sizeof(double) * 64);
   A((void**)&W.ctl, sizeof(int32_t) * 64);
   if (e == cudaSuccess) e = cudaMemset(W.ctl, 0, sizeof(int32_t) * 64);
@@ -541,38 +474,24 @@ void relax_free(RelaxWork& W) {
   W = RelaxWork();
 }
 
-// k iterations of the nine components (every kernel returns at once after
-// the stop).
-// z = M^-1 r (multigrid), z = 0 on fixed unknowns, r.z and beta.
-static pdf_status relax_precondition(pdf_particles* P, int first, cudaStream_t st) {
+static RxSystem relax_system(const pdf_particles* P) {
   const RelaxMesh& R = P->mesh->rx;
-  RelaxWork& W = P->rx;
-  RxDot d;
-  d.wall = R.wall;
-  d.rz = W.scal + kRRz;
-  d.beta = W.scal + kRBeta;
-  d.counter = W.ctl + kRCntUpd;
-  d.first = first;
-  return relax_amg_apply(*W.amg, W.r, W.z, W.ctl + kRActive, W.ctl + kRDone, d, st);
+  const RelaxWork& W = P->rx;
+  RxSystem A;
+  A.n = R.n_rep;
+  A.rp = R.rp; A.ci = R.ci; A.wall = R.wall;
+  A.x = W.x; A.r = W.r; A.z = W.z; A.p = W.p; A.q = W.q;
+  A.part = W.part; A.scal = W.scal; A.ctl = W.ctl;
+  return A;
 }
 
+// k iterations of the nine components (every kernel returns at once after
+// the stop).
 static pdf_status relax_iterations(pdf_particles* P, int k, cudaStream_t st) {
   const RelaxMesh& R = P->mesh->rx;
   RelaxWork& W = P->rx;
   const dim3 grid(W.nb, 9);
-  if (W.multigrid && W.amg) {
-    for (int i = 0; i < k; ++i) {
-      PDF_KERNEL("k_cg_spmv_rec", st, k_cg_spmv_rec<<<grid, kRBlock, 0, st>>>(R.n_rep, R.nnz, R.rp, R.ci, W.aval,
-                                                                               R.wall, W.z, W.p, W.q, W.part, W.scal,
-                                                                               W.ctl));
-      PDF_KERNEL("k_cg_update_mg", st, k_cg_update_mg<<<grid, kRBlock, 0, st>>>(R.n_rep, W.scal, W.x, W.r, W.p, W.q,
-                                                                                 W.part, W.ctl));
-      PDF_KERNEL("k_cg_close", st, k_cg_close<<<1, 32, 0, st>>>(W.ctl));
-      const pdf_status s = relax_precondition(P, 0, st);
-      if (s != PDF_OK) return s;
-    }
-    return PDF_OK;
-  }
+  if (W.multigrid && W.amg) return relax_mg_iterations(*W.amg, relax_system(P), k, st);
   for (int i = 0; i < k; ++i) {
     PDF_KERNEL("k_cg_spmv", st, k_cg_spmv<<<grid, kRBlock, 0, st>>>(R.n_rep, R.nnz, R.rp, R.ci, W.aval, R.wall, W.p,
                                                                      W.q, W.part, W.scal, W.ctl));
@@ -706,17 +625,32 @@ static pdf_status relax_solve(pdf_particles* p, const pdf_model_params* params, 
                                                                    W.p, W.q, W.part));
   PDF_KERNEL("k_cg_reduce", st, k_cg_reduce<<<27, kRBlock, 0, st>>>(W.part, nb, 3, W.scal));
   PDF_KERNEL("k_cg_start", st, k_cg_start<<<1, 32, 0, st>>>(rtol * rtol, max_it, W.scal, W.ctl));
+  bool whole = false;  // the whole solve in one launch
   if (W.multigrid && W.amg) {
-    // the first direction from the multigrid (k_cg_init's Jacobi values
-    // replaced)
     s = relax_amg_values(p, st);
-    if (s == PDF_OK) s = relax_precondition(p, 1, st);
+    if (s != PDF_OK) return s;
+    whole = relax_mg_whole(R.n_rep);
+    if (!whole) s = relax_mg_begin(*W.amg, relax_system(p), st);  // (replaces k_cg_init's Jacobi direction)
     if (s != PDF_OK) return s;
   }
   // iterations in chunks of 8 (CUDA-graph replays while kernel timing is
   // off); the host reads the control words once per chunk
   constexpr int kChunk = 8;
-  if (prof_timing()) {
+  if (whole) {
+    // launches of at most 1,024 iterations, so that no launch runs for long
+    // when the residual stalls above the threshold
+    constexpr int32_t kPerLaunch = 1024;
+    for (int32_t end = std::min(kPerLaunch, max_it);; end += std::min(kPerLaunch, max_it - end)) {
+      s = relax_mg_solve(*W.amg, relax_system(p), end, st);
+      if (s != PDF_OK) return s;
+      if (end >= max_it) break;
+      PDF_CUDA(cudaMemcpyAsync(W.host_ctl, W.ctl, sizeof(int32_t) * 64, cudaMemcpyDeviceToHost, st));
+      PDF_CUDA(cudaStreamSynchronize(st));
+      int left = 0;
+      for (int c = 0; c < 9; ++c) left += W.host_ctl[kRActive + c];
+      if (left == 0) break;
+    }
+  } else if (prof_timing()) {
     for (int launched = 0; launched < max_it; launched += kChunk) {
       s = relax_iterations(p, kChunk, st);
       if (s != PDF_OK) return s;
