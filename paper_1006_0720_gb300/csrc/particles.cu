@@ -223,7 +223,7 @@ static void free_particles(pdf_particles* p) {
   cudaFree(p->u2); cudaFree(p->v2); cudaFree(p->w2); cudaFree(p->om2); cudaFree(p->ps2);
   cudaFree(p->uf2); cudaFree(p->vf2); cudaFree(p->wf2); cudaFree(p->omf2); cudaFree(p->psf2);
   cudaFree(p->pid); cudaFree(p->pid2);
-  cudaFree(p->cond); cudaFree(p->iecm_scratch_f); cudaFree(p->iecm_scratch_i);
+  cudaFree(p->cond); cudaFree(p->iecm_scratch_f); cudaFree(p->iecm_scratch_i); cudaFree(p->iecm_big);
   cudaFree(p->stage);
   double* dbl[] = {p->es, p->ns, p->nd, p->eg, p->nc, p->rows};
   for (double* d : dbl) cudaFree(d);

@@ -209,6 +209,7 @@ extern "C" pdf_status pdf_particles_load(const pdf_mesh* m, const void* buf, siz
     cudaError_t e = cudaMalloc((void**)&P->cond, sizeof(fx::df) * n);
     if (e == cudaSuccess) e = cudaMalloc((void**)&P->iecm_scratch_f, sizeof(float) * 16 * n);
     if (e == cudaSuccess) e = cudaMalloc((void**)&P->iecm_scratch_i, sizeof(int32_t) * 6 * n);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&P->iecm_big, sizeof(int32_t) * ((size_t)P->mesh->d.n_tri + 1));
     if (e != cudaSuccess) s = fail(PDF_ENOMEM, "pdf_particles_load: cudaMalloc failed");
   }
   if (s != PDF_OK) {

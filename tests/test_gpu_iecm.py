@@ -117,3 +117,41 @@ def test_fp32_state_conditional_means():
     s_c = np.bincount(ost["elem"], weights=got, minlength=n_tri)
     s_p = np.bincount(ost["elem"], weights=ost["ps"], minlength=n_tri)
     assert np.allclose(s_c, s_p, rtol=1e-6, atol=1e-6)
+
+
+@pytest.mark.parametrize("precision", [capi.PDF_FP64, capi.PDF_FP32_STATE])
+@pytest.mark.parametrize("values", ["random", "ties", "constant", "wide"])
+def test_conditional_means_at_the_sizes_of_the_sorts(values, precision):
+    """Particle counts at the edges of the per-warp sorts (1, 2, 4 or 8 entries
+    per lane) and above them; velocities that repeat within an element
+    (ordered by particle id), one constant component, values over 60 decades
+    (most of them equal after the sort's linear mapping).  A wrong bin is off
+    by the scalar's spread; right bins by the rounding of a double-float sum."""
+    m = inputs.channel_mesh(8, 6, seed=2)
+    n_tri = len(m["tri"])
+    edges = [1, 2, 3, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 400]
+    counts = np.array([edges[i % len(edges)] for i in range(n_tri)], dtype=np.int32)
+    gm = pg.Mesh(m)
+    gp = pg.Particles(gm, 3, count=counts, u_sigma=0.2, precision=precision)
+    rng = np.random.default_rng(6)
+    st = _host(gp.get_state())
+    n = gp.n
+    for k in ("u", "v", "w"):
+        x = rng.normal(size=n)
+        if values == "ties":
+            x = np.round(x * 4) / 4          # about a dozen values, +0 and -0 among them
+        elif values == "wide":
+            x = x * 10.0 ** rng.integers(-30, 30, n)
+        st[k] = x.astype(np.float32).astype(np.float64)
+    if values == "constant":
+        st["v"][:] = 0.25
+    st["ps"] = rng.random(n).astype(np.float32).astype(np.float64)
+    perm = rng.permutation(n)                # slots in no order, ids not ascending in an element
+    st = {k: np.ascontiguousarray(a[perm]) for k, a in st.items()}
+    gp.set_state({k: torch.from_numpy(a).cuda() for k, a in st.items()})
+    for bins, m_min in (((5, 5, 5), 2), ((7, 3, 9), 1), ((127, 2, 4), 1)):
+        gp.set_iecm(bins, m_min)
+        pg.pdf_estimate_stats(gp, gm)
+        got = gp.iecm_cond().cpu().numpy()
+        want = oracle.iecm_cond(n_tri, st, bins=bins, m_min=m_min)
+        assert np.abs(got - want).max() < 1e-12, (bins, np.abs(got - want).max())
