@@ -284,14 +284,11 @@ struct pdf_particles {
   // grouping
   int32_t* keys[2] = {nullptr, nullptr};
   int32_t* vals[2] = {nullptr, nullptr};
-  int32_t* hist = nullptr;       // [bins][tiles]
-  int32_t* hist_part = nullptr;  // scan partials
+  int32_t* hist = nullptr;       // tile histograms
+  int32_t* hist_part = nullptr;  // digit totals
   int32_t* seg = nullptr;        // [n_tri + 1] segment offsets into the sorted order
   const int32_t* sorted_pid = nullptr;  // storage slot of each sorted position (vals[]), NULL: identity
   int sorted_key_slot = 0;              // keys[] buffer holding the sorted element ids
-  int64_t n_tiles = 0;
-  int64_t hist_len = 0;
-  int32_t n_scan_blocks = 0;
   // counters
   long long* counters = nullptr;  // [16] device
   // elliptic relaxation work space (allocated on first use)

@@ -10,9 +10,6 @@ namespace pdfgb {
 pdf_status estimate_stats_with_buffers(pdf_particles* P, int32_t* keys_a, int32_t* vals_a,
                                        int32_t* keys_b, int32_t* vals_b, int32_t* hist,
                                        int32_t* hist_part, int32_t* seg, cudaStream_t st);
-int64_t radix_tiles(int64_t n);
-int32_t radix_bins();
-int32_t radix_scan_blocks(int64_t hist_len);
 }  // namespace pdfgb
 
 using namespace pdfgb;
@@ -47,9 +44,6 @@ extern "C" pdf_status pdf_estimate_stats_noalloc(pdf_particles* p, const pdf_mes
   if (m->d.n_tri > kMaxElements)
     return fail(PDF_EINVAL, "pdf_estimate_stats_noalloc: " + std::to_string(m->d.n_tri) +
                                 " elements exceed the limit of " + std::to_string(kMaxElements));
-  if (radix_bins() != 512 || radix_tiles(kMaxParticles) != kMaxTiles ||
-      radix_scan_blocks(radix_tiles(p->n) * 512) > kPartInts - 1)
-    return fail(PDF_EINVAL, "pdf_estimate_stats_noalloc: scratch layout does not match the grouping kernels");
   int dev = 0;
   PDF_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return fail(PDF_EINVAL, "pdf_estimate_stats_noalloc: device id out of range");

@@ -9,9 +9,8 @@
 namespace pdfgb {
 
 // Radix grouping geometry (see stats.cu).
-int64_t radix_tiles(int64_t n);
-int32_t radix_bins();
-int32_t radix_scan_blocks(int64_t hist_len);
+int64_t radix_hist_len(int64_t n, int key_bits);
+int32_t radix_part_len();
 
 // One thread per particle.  Particle ids run element by element; elem_off is
 // the exclusive prefix sum of the per-element counts.
@@ -328,16 +327,16 @@ pdf_status alloc_state(pdf_particles* P, cudaStream_t st) {
   SA(P->rows_fx, (int64_t)n_tri);
   SA(P->keys[0], n); SA(P->keys[1], n);
   SA(P->vals[0], n); SA(P->vals[1], n);
-  P->n_tiles = radix_tiles(n);
-  P->hist_len = P->n_tiles * radix_bins();
-  P->n_scan_blocks = radix_scan_blocks(P->hist_len);
-  SA(P->hist, P->hist_len);
-  SA(P->hist_part, P->n_scan_blocks + 1);
+  int key_bits = 1;
+  while ((1LL << key_bits) < (int64_t)n_tri) ++key_bits;
+  SA(P->hist, radix_hist_len(n, key_bits));
+  SA(P->hist_part, radix_part_len());
   SA(P->seg, (int64_t)n_tri + 1);
   SA(P->counters, 16);
   SA(P->pres, n_nodes);
   SA(P->gradP, 2 * (int64_t)n_nodes);
   cudaError_t e = cudaMemsetAsync(P->ns, 0, sizeof(double) * n_nodes * PDF_NNS, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(P->hist_part, 0, sizeof(int32_t) * radix_part_len(), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(P->counters, 0, sizeof(long long) * 16, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(P->pres, 0, sizeof(double) * n_nodes, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(P->gradP, 0, sizeof(double) * 2 * n_nodes, st);

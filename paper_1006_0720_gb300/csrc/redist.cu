@@ -25,9 +25,8 @@ namespace pdfgb {
 pdf_status radix_sort_index(const int32_t* keys, int64_t n, int bits, int32_t* k0, int32_t* v0, int32_t* k1,
                             int32_t* v1, int32_t* hist, int32_t* hist_part, const int32_t** keys_out,
                             const int32_t** vals_out, cudaStream_t st);
-int64_t radix_tiles(int64_t n);
-int32_t radix_bins();
-int32_t radix_scan_blocks(int64_t hist_len);
+int64_t radix_hist_len(int64_t n, int key_bits);
+int32_t radix_part_len();
 
 constexpr int kMaxMin = 64;  // largest min_npel (the critical element's particles fit a warp's scratch)
 
@@ -248,11 +247,18 @@ void redist_free(RedistWork& W) {
   W = RedistWork();
 }
 
+// Bits of an element's particle count.
+static int count_bits(int64_t n) {
+  int bits = 1;
+  while ((1LL << bits) <= n) ++bits;
+  return bits;
+}
+
 static pdf_status redist_alloc(pdf_particles* P) {
   RedistWork& W = P->rd;
   if (W.cnt) return PDF_OK;
   const int64_t nt = P->mesh->d.n_tri;
-  const int64_t hist_len = radix_tiles(nt) * radix_bins();
+  const int64_t hist_len = radix_hist_len(nt, count_bits(P->n));
   cudaError_t e = cudaSuccess;
   auto A = [&](int32_t** p, int64_t n) { if (e == cudaSuccess) e = cudaMalloc((void**)p, sizeof(int32_t) * n); };
   A(&W.cnt, nt);
@@ -261,7 +267,8 @@ static pdf_status redist_alloc(pdf_particles* P) {
   A(&W.k1, nt);
   A(&W.v1, nt);
   A(&W.hist, hist_len);
-  A(&W.hist_part, radix_scan_blocks(hist_len) + 1);
+  A(&W.hist_part, radix_part_len());
+  if (e == cudaSuccess) e = cudaMemset(W.hist_part, 0, sizeof(int32_t) * radix_part_len());
   A(&W.dev, 4);
   A(&W.role, nt);
   A(&W.cur, 2 * nt);
@@ -292,10 +299,8 @@ extern "C" pdf_status pdf_redistribute(pdf_particles* p, const pdf_mesh* m, int3
   PDF_CUDA(cudaMemsetAsync(W.role, 0, sizeof(int32_t) * M.n_tri, st));
   PDF_CUDA(cudaMemsetAsync(W.cur, 0, sizeof(int32_t) * 2 * M.n_tri, st));
   PDF_KERNEL("k_rd_hist", st, k_rd_hist<<<nb, 256, 0, st>>>(p->n, p->elem, W.cnt));
-  int bits = 1;
-  while ((1LL << bits) <= p->n) ++bits;
   const int32_t *sk = nullptr, *sv = nullptr;
-  s = radix_sort_index(W.cnt, M.n_tri, bits, W.k0, W.v0, W.k1, W.v1, W.hist, W.hist_part, &sk, &sv, st);
+  s = radix_sort_index(W.cnt, M.n_tri, count_bits(p->n), W.k0, W.v0, W.k1, W.v1, W.hist, W.hist_part, &sk, &sv, st);
   if (s != PDF_OK) return s;
   PDF_KERNEL("k_rd_nce", st, k_rd_nce<<<1, 32, 0, st>>>(M.n_tri, sk, min_npel, W.dev));
   const int eb = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)M.n_tri + 255) / 256, 4096));

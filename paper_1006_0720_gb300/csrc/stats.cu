@@ -1,11 +1,11 @@
 // Particle-in-cell statistics (sec. 3.3) and derivatives (sec. 3.4).
 //
 // Grouping: a stable least-significant-digit radix sort of (element id,
-// storage slot) pairs, 9-bit digits, in place of the paper's per-element
-// linked lists.  Stability makes the particle order inside every element
-// ascending in storage slot, so the segmented reductions below always add
-// the same numbers in the same order: the statistics are deterministic
-// without floating-point atomics.
+// storage slot) pairs in place of the paper's per-element linked lists.
+// Stability makes the particle order inside every element ascending in
+// storage slot, so the segmented reductions below always add the same
+// numbers in the same order: the statistics are deterministic without
+// floating-point atomics.
 #include <algorithm>
 
 #include "common.cuh"
@@ -13,59 +13,113 @@
 
 namespace pdfgb {
 
-constexpr int kRadixBits = 9;
-constexpr int kBins = 1 << kRadixBits;      // 512
-constexpr int kSortThreads = 256;
-constexpr int kItemsPerThread = 16;
-constexpr int kTile = kSortThreads * kItemsPerThread;  // 4096 keys per tile
+// How a sort of n keys below 2^key_bits is done.  As few passes as digits of
+// up to 11 bits allow, the digits as narrow as that number of passes leaves
+// them: 2,048 elements take one pass, 2^20 (the 535,720-triangle obstacle
+// mesh) two of 10 bits instead of three of 9, and a mesh of 11,000 elements
+// two of 7, whose counters are cheaper to clear and to scan.  Tiles of
+// 2,048 keys instead of 4,096 up to 131,072 keys, so that a small set still
+// spreads over the GPU.  With at most kFusedTiles tiles every scatter block
+// sums the tile counts itself instead of a scan kernel doing so.  Above 8,192
+// tiles, four consecutive tiles share one histogram (a block takes them in
+// turn): the tile counts of 68.6 million keys and 1,024 digits shrink from 68
+// to 17 MB (the scan of them from 42 to 16 us); at 15.9 million keys two tiles
+// per block made the scatter 71 instead of 68 us.
+constexpr int kSortThreads = 256;   // of the histogram
+constexpr int kScatterThreads = 512;
+constexpr int kTileLarge = 4096, kTileSmall = 2048;
+constexpr int kMaxBits = 11, kMinBits = 6;
+constexpr int kFusedTiles = 128;
+struct RadixPlan {
+  int passes, bits, tile;
+  int sub;        // tiles per histogram
+  int64_t tiles;  // histograms
+  bool fused;
+};
+static RadixPlan radix_plan(int64_t n, int key_bits, int max_bits) {
+  RadixPlan R;
+  R.passes = std::max(1, (key_bits + max_bits - 1) / max_bits);
+  R.bits = std::max(kMinBits, (key_bits + R.passes - 1) / R.passes);
+  R.tile = n <= 131072 ? kTileSmall : kTileLarge;
+  R.tiles = (n + R.tile - 1) / R.tile;
+  R.sub = R.tiles > 8192 ? 4 : 1;
+  R.tiles = (R.tiles + R.sub - 1) / R.sub;
+  R.fused = R.tiles <= kFusedTiles;
+  return R;
+}
+static int key_bits_of(int64_t n_keys) {
+  int bits = 1;
+  while ((1LL << bits) < n_keys) ++bits;
+  return bits;
+}
 
-int64_t radix_tiles(int64_t n) { return (n + kTile - 1) / kTile; }
-int32_t radix_bins() { return kBins; }
-// the digit scan runs one block per digit; callers size the partials
-// buffer as radix_scan_blocks(hist_len) + 1
-int32_t radix_scan_blocks(int64_t) { return kBins; }
+// Entries of the tile histogram for n keys below 2^key_bits, and of the digit
+// totals and chunk sums of the scan (any sort; to be zeroed once, every pass
+// that scans leaves the sums at zero again).
+int64_t radix_hist_len(int64_t n, int key_bits) {
+  const RadixPlan R = radix_plan(n, key_bits, kMaxBits);
+  return R.tiles << R.bits;
+}
+constexpr int kScanChunks = 64;  // of tiles
+int32_t radix_part_len() { return (1 + kScanChunks) << kMaxBits; }  // and the chunk sums of the scan
 
-// Per-tile digit histogram, stored bin-major: hist[bin * n_tiles + tile].
-// Thread t counts the tile's keys 16t .. 16t + 15 (four 16-byte loads when
-// the keys are 16-byte aligned) as runs of equal digits, one shared atomic
-// per run: the element ids arrive nearly sorted (the state is reordered
-// by element every few steps, and the second pass reads the first pass's
-// output), so a thread's sixteen keys are mostly one or two runs.
+// Per-tile digit histogram, tile by tile: hist[tile * bins + digit].  (Digit by
+// digit, every count went to a sector of its own: with 10-bit digits the
+// 32-byte sectors of a tile's counts were twice the bytes of its keys, here
+// and again in the scatter.)  Thread t counts the tile's keys PER t ... PER (t + 1) - 1 (16-byte loads when the keys are 16-byte aligned)
+// as runs of equal digits, one shared atomic per run: the element ids arrive
+// nearly sorted (the state is reordered by element every few steps, and the
+// second pass reads the first pass's output), so a thread's keys are mostly
+// one or two runs.  sums (zero before, or NULL): the counts of each chunk of tiles,
+// [kScanChunks][bins], for k_scan_bins.
+// Tiles of chunk c: [n_tiles c / 64, n_tiles (c + 1) / 64); the chunk of a tile.
+__device__ __forceinline__ int64_t scan_chunk(int64_t n_tiles, int64_t tile) {
+  return (kScanChunks * (tile + 1) - 1) / n_tiles;
+}
+template <int BITS, int TILE>
 __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const int32_t* __restrict__ keys, int64_t n,
-                                                             int shift, int64_t n_tiles,
-                                                             int32_t* __restrict__ hist) {
+                                                             int shift, int sub, int32_t* __restrict__ hist,
+                                                             int32_t* __restrict__ sums) {
+  constexpr int kBins = 1 << BITS, kPer = TILE / kSortThreads;
   __shared__ int32_t h[kBins];
   for (int b = threadIdx.x; b < kBins; b += kSortThreads) h[b] = 0;
   __syncthreads();
-  const int64_t i0 = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItemsPerThread;
-  int32_t k[kItemsPerThread];
-  if (i0 + kItemsPerThread <= n && (reinterpret_cast<uintptr_t>(keys + i0) & 15) == 0) {
-    const int4* q = reinterpret_cast<const int4*>(keys + i0);
+  for (int t = 0; t < sub; ++t) {
+    const int64_t i0 = ((int64_t)blockIdx.x * sub + t) * TILE + (int64_t)threadIdx.x * kPer;
+    int32_t k[kPer];
+    if (i0 + kPer <= n && (reinterpret_cast<uintptr_t>(keys + i0) & 15) == 0) {
+      const int4* q = reinterpret_cast<const int4*>(keys + i0);
 #pragma unroll
-    for (int j = 0; j < kItemsPerThread / 4; ++j) {
-      const int4 v = __ldg(q + j);
-      k[4 * j] = v.x; k[4 * j + 1] = v.y; k[4 * j + 2] = v.z; k[4 * j + 3] = v.w;
+      for (int j = 0; j < kPer / 4; ++j) {
+        const int4 v = __ldg(q + j);
+        k[4 * j] = v.x; k[4 * j + 1] = v.y; k[4 * j + 2] = v.z; k[4 * j + 3] = v.w;
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < kPer; ++r) k[r] = (i0 + r < n) ? __ldg(keys + i0 + r) : 0;
     }
-  } else {
+    const int m = (int)max((int64_t)0, min((int64_t)kPer, n - i0));  // keys of this thread
+    int run_d = -1, run_c = 0;
 #pragma unroll
-    for (int r = 0; r < kItemsPerThread; ++r) k[r] = (i0 + r < n) ? __ldg(keys + i0 + r) : 0;
-  }
-  const int m = (int)max((int64_t)0, min((int64_t)kItemsPerThread, n - i0));  // keys of this thread
-  int run_d = -1, run_c = 0;
-#pragma unroll
-  for (int r = 0; r < kItemsPerThread; ++r) {
-    if (r >= m) break;
-    const int d = (k[r] >> shift) & (kBins - 1);
-    if (d != run_d) {
-      if (run_c) atomicAdd(&h[run_d], run_c);
-      run_d = d;
-      run_c = 0;
+    for (int r = 0; r < kPer; ++r) {
+      if (r >= m) break;
+      const int d = (k[r] >> shift) & (kBins - 1);
+      if (d != run_d) {
+        if (run_c) atomicAdd(&h[run_d], run_c);
+        run_d = d;
+        run_c = 0;
+      }
+      ++run_c;
     }
-    ++run_c;
+    if (run_c) atomicAdd(&h[run_d], run_c);
   }
-  if (run_c) atomicAdd(&h[run_d], run_c);
   __syncthreads();
-  for (int b = threadIdx.x; b < kBins; b += kSortThreads) hist[(int64_t)b * n_tiles + blockIdx.x] = h[b];
+  if (sums) sums += scan_chunk(gridDim.x, blockIdx.x) * kBins;
+  for (int b = threadIdx.x; b < kBins; b += kSortThreads) {
+    const int32_t c = h[b];
+    hist[(int64_t)blockIdx.x * kBins + b] = c;
+    if (sums && c) atomicAdd(sums + b, c);
+  }
 }
 
 // Exclusive block-wide prefix sum (blockDim a multiple of 32, at most
@@ -99,129 +153,212 @@ __device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t* tota
   return r;
 }
 
-// Per digit, one block each: the exclusive prefix of the digit's tile
-// counts over the tiles (in place; the digit's row of hist is contiguous)
-// and the digit's total in part[digit].  The scatter adds the totals of the
-// smaller digits.  512 threads (the 512 digit blocks fit on the GPU at once,
-// four per SM); each round stages 4,096 entries through shared memory with
-// coalesced loads and stores, thread t scanning entries 8t .. 8t + 7 (one
-// padding word per 32 keeps those reads free of bank conflicts).
-constexpr int kScanThreads = 512;
-constexpr int kScanPer = 8;
-constexpr int kScanRound = kScanThreads * kScanPer;  // 4096
-__device__ __forceinline__ int scan_pad(int i) { return i + (i >> 5); }
-__global__ void __launch_bounds__(kScanThreads, 4) k_scan_bins(int32_t* __restrict__ hist, int64_t n_tiles,
-                                                            int32_t* __restrict__ part) {
-  __shared__ int32_t s[kScanRound + kScanRound / 32];
-  int32_t* row = hist + (int64_t)blockIdx.x * n_tiles;
-  int32_t carry = 0;
-  for (int64_t start = 0; start < n_tiles; start += kScanRound) {
+// The exclusive prefix of every digit's counts over the tiles, in place, and
+// the digits' totals in part, by blocks of a chunk of tiles (blockIdx.x) and a
+// group of 32 digits (blockIdx.y), from the sums of the earlier chunks.
+// Thread (x, y) takes digit x of the group and the y-th of the chunk's eight
+// runs of tiles, so that a warp reads 128 consecutive bytes.
+__global__ void __launch_bounds__(256) k_scan_bins(int32_t* __restrict__ hist, int64_t n_tiles, int bins,
+                                                   const int32_t* __restrict__ sums, int32_t* __restrict__ part) {
+  __shared__ int32_t before[8][32], own[8][32];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5, b = blockIdx.y * 32 + x;
+  const int64_t c0 = n_tiles * blockIdx.x / kScanChunks, c1 = n_tiles * (blockIdx.x + 1) / kScanChunks;
+  const int64_t lo = c0 + (c1 - c0) * y / 8, hi = c0 + (c1 - c0) * (y + 1) / 8;
+  int32_t t = 0, p = 0;
 #pragma unroll
-    for (int j = 0; j < kScanPer; ++j) {
-      const int i = threadIdx.x + j * kScanThreads;
-      s[scan_pad(i)] = (start + i < n_tiles) ? row[start + i] : 0;
-    }
-    __syncthreads();
-    int32_t v[kScanPer];
-    int32_t sum = 0;
-#pragma unroll
-    for (int j = 0; j < kScanPer; ++j) {
-      v[j] = s[scan_pad(kScanPer * threadIdx.x + j)];
-      sum += v[j];
-    }
-    int32_t total;
-    int32_t ex = block_exclusive_scan(sum, &total) + carry;  // (its barriers order the reads above)
-#pragma unroll
-    for (int j = 0; j < kScanPer; ++j) {
-      s[scan_pad(kScanPer * threadIdx.x + j)] = ex;
-      ex += v[j];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < kScanPer; ++j) {
-      const int i = threadIdx.x + j * kScanThreads;
-      if (start + i < n_tiles) row[start + i] = s[scan_pad(i)];
-    }
-    carry += total;
-    __syncthreads();  // the next round overwrites s
+  for (int c = y; c < kScanChunks; c += 8) {  // the chunks before this one, and all
+    const int32_t v = __ldg(sums + c * bins + b);
+    if (c < (int)blockIdx.x) p += v;
+    t += v;
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = carry;
+  before[y][x] = p;
+  own[y][x] = t;
+  __syncthreads();
+  if (blockIdx.x == 0 && y == 0) {
+    int32_t total = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) total += own[k][x];
+    part[b] = total;
+  }
+  __syncthreads();
+  t = 0;
+#pragma unroll 4
+  for (int64_t i = lo; i < hi; ++i) t += hist[i * bins + b];
+  own[y][x] = t;
+  __syncthreads();
+  int32_t acc = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) acc += before[k][x] + (k < y ? own[k][x] : 0);
+#pragma unroll 4
+  for (int64_t i = lo; i < hi; ++i) {
+    const int32_t v = hist[i * bins + b];
+    hist[i * bins + b] = acc;
+    acc += v;
+  }
 }
 
-// Stable scatter of one tile, 512 threads of 8 items.  Warp w owns the
-// tile's items [256 w, 256 (w + 1)) and ranks them in 8 rounds of 32 in
+// Stable scatter of `sub` consecutive tiles, one after the other, by 512
+// threads.  Warp w owns the tile's items
+// [TILE / 16 w, TILE / 16 (w + 1)) and ranks them in rounds of 32 in
 // index order (match.any groups equal digits, one lane of each group
 // advances the warp's own row of shared digit counters, so no block barrier
 // between rounds); one pass over the (warp, digit) counts then gives every
 // warp and digit its output offset, so items with equal digits keep their
-// index order.  Twice the warps per SM of 256 threads with 16 items each
-// (64 registers, two blocks per SM): the ranking waits on the MIO queue, and
-// more warps cover it.
-constexpr int kScatterThreads = 512;
-constexpr int kScatterItems = kTile / kScatterThreads;  // 8
-__global__ void __launch_bounds__(kScatterThreads, 2) k_radix_scatter(
+// index order.  The digits' bases come from the scanned histogram (hist, part)
+// or (FUSED) from the unscanned one.  seg (a single-pass sort by
+// element): block 0 also writes the segment offsets, which are the digit
+// bases.  Tiles of 4,096 keys and digits of 9 bits: 64 registers, two blocks
+// per SM; the ranking waits on the MIO queue, and more warps (512 threads of 8
+// items instead of 256 of 16) cover it.
+template <int BITS>
+constexpr size_t scatter_shared() {
+  return sizeof(int32_t) * ((size_t)(kScatterThreads / 32) * ((1 << BITS) + 1) + (1 << BITS));
+}
+template <int BITS, int TILE, bool FUSED>
+__global__ void __launch_bounds__(kScatterThreads, BITS <= 10 ? 2 : 1) k_radix_scatter(
     const int32_t* __restrict__ keys_in, const int32_t* __restrict__ vals_in, int64_t n, int shift,
-    int64_t n_tiles, const int32_t* __restrict__ hist, const int32_t* __restrict__ part,
-    int32_t* __restrict__ keys_out, int32_t* __restrict__ vals_out) {
-  constexpr int kWarps = kScatterThreads / 32;  // 16
-  constexpr int kPerWarp = kTile / kWarps;      // 256 items, 8 rounds
-  static_assert(kBins == kScatterThreads, "one digit per thread in the digit-base scan");
-  __shared__ int32_t wcnt[kWarps][kBins + 1];  // the extra bin takes the tile's padding
-  __shared__ int32_t dbase[kBins];             // first output position of each digit
+    int sub, int64_t n_tiles, const int32_t* __restrict__ hist, int32_t* __restrict__ part,
+    int32_t* __restrict__ keys_out, int32_t* __restrict__ vals_out, int32_t* __restrict__ seg, int32_t n_seg) {
+  constexpr int kBins = 1 << BITS;
+  constexpr int kWarps = kScatterThreads / 32;       // 16
+  constexpr int kPerWarp = TILE / kWarps;            // 256 or 128 items
+  constexpr int kItems = kPerWarp / 32;              // 8 or 4 rounds
+  constexpr int kDig = kBins > kScatterThreads ? kBins / kScatterThreads : 1;  // digits per thread
+  extern __shared__ __align__(16) int32_t smem[];
+  int32_t* wcnt = smem;                              // [kWarps][kBins + 1]; the extra bin takes the tile's padding
+  int32_t* dbase = smem + kWarps * (kBins + 1);      // [kBins] next output position of each digit
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  {
-    const int32_t c0 = __ldg(part + threadIdx.x);
-    int32_t total;
-    dbase[threadIdx.x] = block_exclusive_scan(c0, &total);
+  int64_t w0 = (int64_t)blockIdx.x * sub * TILE + (int64_t)wid * kPerWarp;
+  int32_t key[kItems], val[kItems], off[kItems];
+  auto load = [&]() {
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+      const int64_t i = w0 + r * 32 + lane;
+      const bool valid = i < n;
+      key[r] = valid ? keys_in[i] : 0;
+      val[r] = valid ? (vals_in ? vals_in[i] : (int32_t)i) : 0;
+    }
+  };
+  load();
+  // the counts of the thread's digits in the earlier tiles and in all tiles
+  const int b0 = threadIdx.x * kDig;
+  int32_t mine[kDig], total[kDig];
+#pragma unroll
+  for (int q = 0; q < kDig; ++q) mine[q] = total[q] = 0;
+  if (FUSED) {
+    // 512 / bins threads share a digit below 512 bins, each every so many tiles
+    constexpr int kShare = kBins < kScatterThreads ? kScatterThreads / kBins : 1;
+    const int d0 = kShare > 1 ? threadIdx.x % kBins : b0;
+    const int t0 = kShare > 1 ? threadIdx.x / kBins : 0;
+#pragma unroll 8
+    for (int t = t0; t < (int)n_tiles; t += kShare) {
+      int32_t c[kDig];
+      const int32_t* h = hist + (int64_t)t * kBins + d0;
+      if (kDig == 4) {
+        const int4 v = __ldg(reinterpret_cast<const int4*>(h));
+        c[0] = v.x; c[kDig - 3] = v.y; c[kDig - 2] = v.z; c[kDig - 1] = v.w;
+      } else {
+#pragma unroll
+        for (int q = 0; q < kDig; ++q) c[q] = __ldg(h + q);
+      }
+#pragma unroll
+      for (int q = 0; q < kDig; ++q) {
+        total[q] += c[q];
+        if (t < (int)blockIdx.x) mine[q] += c[q];
+      }
+    }
+    if (kShare > 1) {  // (kDig == 1; the counters' space for the shares)
+      wcnt[threadIdx.x] = mine[0];
+      wcnt[kScatterThreads + threadIdx.x] = total[0];
+      __syncthreads();
+      mine[0] = total[0] = 0;
+      if (b0 < kBins) {
+#pragma unroll
+        for (int k = 0; k < kShare; ++k) {
+          mine[0] += wcnt[k * kBins + b0];
+          total[0] += wcnt[kScatterThreads + k * kBins + b0];
+        }
+      }
+      __syncthreads();
+    }
+  } else if (b0 < kBins) {
+#pragma unroll
+    for (int q = 0; q < kDig; ++q) {
+      total[q] = __ldg(part + b0 + q);
+      mine[q] = hist[(int64_t)blockIdx.x * kBins + b0 + q];
+    }
+    // the chunk sums behind part go back to zero for the next pass
+    if (blockIdx.x < kScanChunks) {
+#pragma unroll
+      for (int q = 0; q < kDig; ++q) part[(1 + blockIdx.x) * kBins + b0 + q] = 0;
+    }
   }
-  // this tile's count of the thread's digit, loaded before the ranking
-  const int32_t th0 = hist[(int64_t)threadIdx.x * n_tiles + blockIdx.x];
-  for (int i = threadIdx.x; i < kWarps * (kBins + 1); i += kScatterThreads) (&wcnt[0][0])[i] = 0;
+  for (int i = threadIdx.x; i < kWarps * (kBins + 1); i += kScatterThreads) wcnt[i] = 0;
+  {
+    int32_t sum = 0;
+#pragma unroll
+    for (int q = 0; q < kDig; ++q) sum += total[q];
+    int32_t all;
+    int32_t base = block_exclusive_scan(sum, &all);
+#pragma unroll
+    for (int q = 0; q < kDig; ++q) {
+      if (b0 < kBins) {
+        dbase[b0 + q] = base + mine[q];
+        if (seg && blockIdx.x == 0 && b0 + q < n_seg) seg[b0 + q] = base;
+      }
+      base += total[q];
+    }
+    if (seg && blockIdx.x == 0 && threadIdx.x == 0) seg[n_seg] = (int32_t)n;
+  }
   __syncthreads();
   const uint32_t lt_mask = (1u << lane) - 1u;
-  const int64_t w0 = (int64_t)blockIdx.x * kTile + (int64_t)wid * kPerWarp;
-  int32_t key[kScatterItems], val[kScatterItems], off[kScatterItems];
+  int32_t* row = wcnt + wid * (kBins + 1);
+  for (int t = 0;;) {
 #pragma unroll
-  for (int r = 0; r < kScatterItems; ++r) {
-    const int64_t i = w0 + r * 32 + lane;
-    const bool valid = i < n;
-    key[r] = valid ? keys_in[i] : 0;
-    val[r] = valid ? (vals_in ? vals_in[i] : (int32_t)i) : 0;
-  }
-#pragma unroll
-  for (int r = 0; r < kScatterItems; ++r) {
+  for (int r = 0; r < kItems; ++r) {
     const int64_t i = w0 + r * 32 + lane;
     const int d = (i < n) ? ((key[r] >> shift) & (kBins - 1)) : kBins;
     const uint32_t peers = __match_any_sync(0xffffffffu, d);
     const int rank = __popc(peers & lt_mask);
-    const int32_t before = wcnt[wid][d];
+    const int32_t before = row[d];
     __syncwarp();
-    if (rank == 0) wcnt[wid][d] = before + __popc(peers);
+    if (rank == 0) row[d] = before + __popc(peers);
     __syncwarp();
     off[r] = before + rank;
   }
   __syncthreads();
-  {  // (warp, digit) offsets: the digit's base, the earlier tiles' counts of
-     // the digit and the earlier warps' counts
-    const int b = threadIdx.x;
-    int32_t acc = dbase[b] + th0;
+  // (warp, digit) offsets: the digit's next position and the earlier warps' counts
+#pragma unroll
+  for (int q = 0; q < kDig; ++q) {
+    const int b = b0 + q;
+    if (b >= kBins) break;
+    int32_t acc = dbase[b];
 #pragma unroll
     for (int k = 0; k < kWarps; ++k) {
-      const int32_t c = wcnt[k][b];
-      wcnt[k][b] = acc;
+      const int32_t c = wcnt[k * (kBins + 1) + b];
+      wcnt[k * (kBins + 1) + b] = acc;
       acc += c;
     }
+    dbase[b] = acc;
   }
   __syncthreads();
 #pragma unroll
-  for (int r = 0; r < kScatterItems; ++r) {
+  for (int r = 0; r < kItems; ++r) {
     const int64_t i = w0 + r * 32 + lane;
     if (i < n) {
       const int d = (key[r] >> shift) & (kBins - 1);
-      const int32_t pos = wcnt[wid][d] + off[r];
+      const int32_t pos = row[d] + off[r];
       keys_out[pos] = key[r];
       vals_out[pos] = val[r];
     }
+  }
+  if (++t == sub) break;
+  // the block's next tile
+  w0 += TILE;
+  load();
+  __syncthreads();
+  for (int i = threadIdx.x; i < kWarps * (kBins + 1); i += kScatterThreads) wcnt[i] = 0;
+  __syncthreads();
   }
 }
 
@@ -578,15 +715,66 @@ static int blocks_for(int64_t n, int threads) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)sm_count() * 32));
 }
 
-// One stable pass of the radix sort on the digit at `shift`: tile
-// histograms, the per-digit scan over the tiles, the scatter.  hist holds
-// n_tiles * kBins entries, part kBins.
-static pdf_status radix_pass(const int32_t* kin, const int32_t* vin, int64_t n, int shift, int64_t n_tiles,
-                             int32_t* hist, int32_t* part, int32_t* kout, int32_t* vout, cudaStream_t st) {
-  PDF_KERNEL("k_radix_hist", st, k_radix_hist<<<(unsigned)n_tiles, kSortThreads, 0, st>>>(kin, n, shift, n_tiles, hist););
-  PDF_KERNEL("k_scan_bins", st, k_scan_bins<<<kBins, kScanThreads, 0, st>>>(hist, n_tiles, part););
-  PDF_KERNEL("k_radix_scatter", st, k_radix_scatter<<<(unsigned)n_tiles, kScatterThreads, 0, st>>>(
-                                        kin, vin, n, shift, n_tiles, hist, part, kout, vout););
+// One stable pass of the radix sort on the digit at `shift` (see RadixPlan).
+template <int BITS, int TILE, bool FUSED>
+static pdf_status radix_pass_t(const RadixPlan& R, const int32_t* kin, const int32_t* vin, int64_t n, int shift,
+                               int32_t* hist, int32_t* part, int32_t* kout, int32_t* vout, int32_t* seg,
+                               int32_t n_seg, cudaStream_t st) {
+  const unsigned nt = (unsigned)R.tiles;
+  constexpr size_t bytes = scatter_shared<BITS>();
+  if (bytes > 48 * 1024)
+    PDF_CUDA(cudaFuncSetAttribute(k_radix_scatter<BITS, TILE, FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)bytes));
+  constexpr int kBins = 1 << BITS;
+  int32_t* sums = FUSED ? nullptr : part + kBins;
+  PDF_KERNEL("k_radix_hist", st, k_radix_hist<BITS, TILE><<<nt, kSortThreads, 0, st>>>(kin, n, shift, R.sub, hist, sums););
+  if (!FUSED)
+    PDF_KERNEL("k_scan_bins", st, k_scan_bins<<<dim3(kScanChunks, kBins / 32), 256, 0, st>>>(hist, R.tiles, kBins, sums, part););
+  PDF_KERNEL("k_radix_scatter", st, k_radix_scatter<BITS, TILE, FUSED><<<nt, kScatterThreads, bytes, st>>>(
+                                        kin, vin, n, shift, R.sub, R.tiles, hist, part, kout, vout, seg, n_seg););
+  return PDF_OK;
+}
+template <int BITS>
+static pdf_status radix_pass_b(const RadixPlan& R, const int32_t* kin, const int32_t* vin, int64_t n, int shift,
+                               int32_t* hist, int32_t* part, int32_t* kout, int32_t* vout, int32_t* seg,
+                               int32_t n_seg, cudaStream_t st) {
+  if (R.tile == kTileSmall)  // (at most 64 tiles: always fused)
+    return radix_pass_t<BITS, kTileSmall, true>(R, kin, vin, n, shift, hist, part, kout, vout, seg, n_seg, st);
+  if (R.fused)
+    return radix_pass_t<BITS, kTileLarge, true>(R, kin, vin, n, shift, hist, part, kout, vout, seg, n_seg, st);
+  return radix_pass_t<BITS, kTileLarge, false>(R, kin, vin, n, shift, hist, part, kout, vout, seg, n_seg, st);
+}
+static pdf_status radix_pass(const RadixPlan& R, const int32_t* kin, const int32_t* vin, int64_t n, int shift,
+                             int32_t* hist, int32_t* part, int32_t* kout, int32_t* vout, int32_t* seg,
+                             int32_t n_seg, cudaStream_t st) {
+  switch (R.bits) {
+    case 6: return radix_pass_b<6>(R, kin, vin, n, shift, hist, part, kout, vout, seg, n_seg, st);
+    case 7: return radix_pass_b<7>(R, kin, vin, n, shift, hist, part, kout, vout, seg, n_seg, st);
+    case 8: return radix_pass_b<8>(R, kin, vin, n, shift, hist, part, kout, vout, seg, n_seg, st);
+    case 9: return radix_pass_b<9>(R, kin, vin, n, shift, hist, part, kout, vout, seg, n_seg, st);
+    case 10: return radix_pass_b<10>(R, kin, vin, n, shift, hist, part, kout, vout, seg, n_seg, st);
+    default: return radix_pass_b<11>(R, kin, vin, n, shift, hist, part, kout, vout, seg, n_seg, st);
+  }
+}
+
+// Stable grouping by element of n keys into the last of the passes' buffers
+// (kout[pass], vout[pass]) with the segment offsets in seg.
+static pdf_status group_keys(const RadixPlan& R, const int32_t* elem, int64_t n, int32_t n_tri, int32_t* hist,
+                             int32_t* part, int32_t* const* kout, int32_t* const* vout, int32_t* seg,
+                             cudaStream_t st) {
+  const int32_t* kin = elem;
+  const int32_t* vin = nullptr;  // first pass: the values are the indices
+  const bool one = R.passes == 1;
+  for (int pass = 0; pass < R.passes; ++pass) {
+    const pdf_status s = radix_pass(R, kin, vin, n, pass * R.bits, hist, part, kout[pass], vout[pass],
+                                    one ? seg : nullptr, n_tri, st);
+    if (s != PDF_OK) return s;
+    kin = kout[pass];
+    vin = vout[pass];
+  }
+  if (!one)
+    PDF_KERNEL("k_seg_offsets", st, k_seg_offsets<<<(unsigned)((seg_offsets_threads(n) + 255) / 256), 256, 0, st>>>(
+                                        kin, n, n_tri, seg););
   return PDF_OK;
 }
 
@@ -594,25 +782,13 @@ static pdf_status radix_pass(const int32_t* kin, const int32_t* vin, int64_t n, 
 // keys[out], particle ids in vals[out] and segment offsets in seg.
 pdf_status group_by_element(pdf_particles* P, cudaStream_t st) {
   const int32_t n_tri = P->mesh->d.n_tri;
-  const int64_t n = P->n;
-  int bits = 1;
-  while ((1LL << bits) < (int64_t)n_tri) ++bits;
-  const int passes = (bits + kRadixBits - 1) / kRadixBits;
-  const int32_t* kin = P->elem;
-  const int32_t* vin = nullptr;  // first pass: particle ids are the indices
-  int cur = 0;
-  for (int pass = 0; pass < passes; ++pass) {
-    const int shift = pass * kRadixBits;
-    const pdf_status s = radix_pass(kin, vin, n, shift, P->n_tiles, P->hist, P->hist_part, P->keys[cur],
-                                    P->vals[cur], st);
-    if (s != PDF_OK) return s;
-    kin = P->keys[cur];
-    vin = P->vals[cur];
-    cur ^= 1;
-  }
-  PDF_KERNEL("k_seg_offsets", st, k_seg_offsets<<<(unsigned)((seg_offsets_threads(n) + 255) / 256), 256, 0, st>>>(kin, n, n_tri, P->seg););
-  P->sorted_pid = vin;
-  P->sorted_key_slot = cur ^ 1;
+  const RadixPlan R = radix_plan(P->n, key_bits_of(n_tri), kMaxBits);
+  int32_t* const kout[3] = {P->keys[0], P->keys[1], P->keys[0]};
+  int32_t* const vout[3] = {P->vals[0], P->vals[1], P->vals[0]};
+  const pdf_status s = group_keys(R, P->elem, P->n, n_tri, P->hist, P->hist_part, kout, vout, P->seg, st);
+  if (s != PDF_OK) return s;
+  P->sorted_key_slot = (R.passes - 1) & 1;
+  P->sorted_pid = P->vals[P->sorted_key_slot];
   return PDF_OK;
 }
 
@@ -766,32 +942,22 @@ extern "C" pdf_status pdf_estimate_stats(pdf_particles* p, const pdf_mesh* m, do
 namespace pdfgb {
 
 // Statistics with caller-chosen grouping buffers (used by the
-// allocation-free entry point in noalloc.cu).  keys_a/vals_a receive the
-// first radix pass, keys_b/vals_b the second; at most two passes, so
-// n_tri <= 2^18.
+// allocation-free entry point in noalloc.cu).  keys_b/vals_b receive the
+// result; at most two passes of 9-bit digits, so n_tri <= 2^18; hist holds
+// 512 entries per 4,096 keys, and the tile counts are never scanned (at most
+// 128 tiles).
 pdf_status estimate_stats_with_buffers(pdf_particles* P, int32_t* keys_a, int32_t* vals_a,
                                        int32_t* keys_b, int32_t* vals_b, int32_t* hist,
                                        int32_t* hist_part, int32_t* seg, cudaStream_t st) {
   const MeshDev& M = P->mesh->d;
-  const int64_t n = P->n;
-  int bits = 1;
-  while ((1LL << bits) < (int64_t)M.n_tri) ++bits;
-  const int passes = (bits + kRadixBits - 1) / kRadixBits;
-  if (passes > 2) return fail(PDF_EINVAL, "estimate_stats_with_buffers: more than 2^18 elements");
-  const int64_t n_tiles = radix_tiles(n);
-  const int32_t* kin = P->elem;
-  const int32_t* vin = nullptr;
-  int32_t* kout[2] = {passes == 2 ? keys_a : keys_b, keys_b};
-  int32_t* vout[2] = {passes == 2 ? vals_a : vals_b, vals_b};
-  for (int pass = 0; pass < passes; ++pass) {
-    const int shift = pass * kRadixBits;
-    const pdf_status s = radix_pass(kin, vin, n, shift, n_tiles, hist, hist_part, kout[pass], vout[pass], st);
-    if (s != PDF_OK) return s;
-    kin = kout[pass];
-    vin = vout[pass];
-  }
-  PDF_KERNEL("k_seg_offsets", st, k_seg_offsets<<<(unsigned)((seg_offsets_threads(n) + 255) / 256), 256, 0, st>>>(kin, n, M.n_tri, seg));
-  pdf_status s = elem_stats(P, seg, vin, st);
+  const RadixPlan R = radix_plan(P->n, key_bits_of(M.n_tri), 9);
+  if (R.passes > 2) return fail(PDF_EINVAL, "estimate_stats_with_buffers: more than 2^18 elements");
+  int32_t* const kout[2] = {R.passes == 2 ? keys_a : keys_b, keys_b};
+  int32_t* const vout[2] = {R.passes == 2 ? vals_a : vals_b, vals_b};
+  pdf_status s = group_keys(R, P->elem, P->n, M.n_tri, hist, hist_part, kout, vout, seg, st);
+  if (s != PDF_OK) return s;
+  const int32_t* vin = vals_b;
+  s = elem_stats(P, seg, vin, st);
   if (s != PDF_OK) return s;
   s = node_stats_from_elements(P, st);
   if (s != PDF_OK) return s;
@@ -801,23 +967,21 @@ pdf_status estimate_stats_with_buffers(pdf_particles* P, int32_t* keys_a, int32_
 
 // Stable LSD radix sort of n non-negative int32 keys below 2^bits, the
 // values the original indices; ping-pong buffers k0/v0, k1/v1 of n entries,
-// hist of radix_tiles(n) * radix_bins() and hist_part of
-// radix_scan_blocks(hist_len) + 1 entries.  *keys_out / *vals_out receive
-// the sorted buffers.
+// hist of radix_hist_len(n, bits) and hist_part of radix_part_len() entries,
+// zeroed once.
+// *keys_out / *vals_out receive the sorted buffers.
 pdf_status radix_sort_index(const int32_t* keys, int64_t n, int bits, int32_t* k0, int32_t* v0, int32_t* k1,
                             int32_t* v1, int32_t* hist, int32_t* hist_part, const int32_t** keys_out,
                             const int32_t** vals_out, cudaStream_t st) {
-  const int64_t n_tiles = radix_tiles(n);
-  const int passes = std::max(1, (bits + kRadixBits - 1) / kRadixBits);
+  const RadixPlan R = radix_plan(n, bits, kMaxBits);
   const int32_t* kin = keys;
   const int32_t* vin = nullptr;
   int32_t* kout[2] = {k0, k1};
   int32_t* vout[2] = {v0, v1};
-  for (int pass = 0; pass < passes; ++pass) {
-    const int shift = pass * kRadixBits;
+  for (int pass = 0; pass < R.passes; ++pass) {
     int32_t* ko = kout[pass & 1];
     int32_t* vo = vout[pass & 1];
-    const pdf_status s = radix_pass(kin, vin, n, shift, n_tiles, hist, hist_part, ko, vo, st);
+    const pdf_status s = radix_pass(R, kin, vin, n, pass * R.bits, hist, hist_part, ko, vo, nullptr, 0, st);
     if (s != PDF_OK) return s;
     kin = ko;
     vin = vo;
