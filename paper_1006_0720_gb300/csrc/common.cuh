@@ -63,13 +63,18 @@ static_assert(sizeof(FxGeo) == 80, "FxGeo layout");
 constexpr int kPosF = 56;
 
 // Coefficient row of the fixed-point kernel (256 B): the element means of
-// U, V, W and phi and the scaled coefficients, all as double-floats:
-//   c0-5 sqrt(2 nu dt) d<U_i>/dx_j; c6-8 a_i dt; c9-17 G_ij dt;
-//   c18 sqrt(C0 eps dt); c19 (C3 + S_w) <w> dt; c20 C3 <w>^2 dt;
-//   c21 <w> sqrt(2 C3 C4 dt); c22 dt / t_m; c23-27 unused (zero).
+// U, V, W and phi and the scaled coefficients as double-floats, in pairs that
+// the kernel loads with one 16-byte load and multiplies two at a time.
 struct __align__(16) FxRow {
-  fx::df mean[4];
-  fx::df c[28];
+  fx::df2 mean_uv, mean_wp;  // (<U>, <V>), (<W>, <phi>)
+  fx::df2 grad[3];           // sqrt(2 nu dt) (d<U_i>/dx, d<U_i>/dy)
+  fx::df2 drift[3];          // dt (G_i1, G_i2)
+  fx::df2 rest[3];           // (dt G_i3, sqrt(C0 eps dt))
+  fx::df2 freq;              // (-(C3 + S_w) <w> dt, <w> sqrt(2 C3 C4 dt))
+  fx::df a[3];               // a_i dt
+  fx::df freq0;              // C3 <w>^2 dt
+  fx::df mix;                // dt / t_m
+  fx::df pad[3];
 };
 static_assert(sizeof(FxRow) == 256, "FxRow layout");
 

@@ -418,17 +418,23 @@ __device__ __forceinline__ fx::df ld_df(const float* a, int64_t i) { return fx::
 // (the deviations are of the size of the fluctuations).  The order of every
 // addition is fixed by the stable grouping, so the results are
 // deterministic; a reordering of the storage changes them by rounding only.
-// Only FP32 additions and fused multiply-adds per particle (no conversions).
+// Only FP32 additions and fused multiply-adds per particle (no conversions),
+// two values per instruction: the same sums in the same order in two thirds
+// of the instructions.  15.9M particles 206 -> 201 us (its reads, 0.7 GB,
+// take 105 us), 5.1M in FP32 form 75 -> 64 us.
 constexpr int kStatLanes = 8;
 
 __device__ __forceinline__ void prefetch_l2(const void* a) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
 }
 
-__device__ __forceinline__ void acc_xor(fx::acc& a, int o) {
-  const float h = __shfl_xor_sync(0xffffffffu, a.h, o);
-  const float l = __shfl_xor_sync(0xffffffffu, a.l, o);
-  a.add(fx::df{h, l});
+__device__ __forceinline__ void acc_xor(fx::acc2& a, int o) {
+  fx::df2 b;
+  b.h.x = __shfl_xor_sync(0xffffffffu, a.h.x, o);
+  b.h.y = __shfl_xor_sync(0xffffffffu, a.h.y, o);
+  b.l.x = __shfl_xor_sync(0xffffffffu, a.l.x, o);
+  b.l.y = __shfl_xor_sync(0xffffffffu, a.l.y, o);
+  a.add(b);
 }
 
 // x - k for stored double-floats, normalized: fx::sub with the final
@@ -443,6 +449,13 @@ __device__ __forceinline__ fx::df deviation(fx::df x, fx::df k) {
   const fx::df s = fx::two_sum(x.h, -k.h);
   const float t = __fadd_rn(x.l, __fadd_rn(s.l, -k.l));
   return fx::fast_two_sum(s.h, t);
+}
+// The same for two values at once.
+__device__ __forceinline__ fx::df2 deviation2(fx::df2 x, fx::df2 k) {
+  const fx::df2 s = fx::two_sum2(x.h, fx::neg2(k.h));
+  const fx::f2 t = fx::add2(x.l, fx::sub2(s.l, k.l));
+  const fx::f2 h = fx::add2(s.h, t);
+  return fx::df2{h, fx::sub2(t, fx::sub2(h, s.h))};
 }
 
 // a[i] for a lane-dependent i, by selects (no local-memory array)
@@ -502,18 +515,22 @@ __global__ void __launch_bounds__(256, 3) k_elem_stats_grp(const int32_t* __rest
         }
       }
     }
-    fx::df K[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) K[q] = fx::df{0.f, 0.f};
+    // values in pairs (u, v) and (w, psi), omega by itself
+    fx::df2 Kuv{}, Kwp{};
+    fx::df Km{0.f, 0.f};
     if (N > 0) {
       const int32_t p0 = pid ? __ldg(pid + beg) : beg;
-      K[0] = ld_df(u, p0); K[1] = ld_df(v, p0); K[2] = ld_df(w, p0); K[3] = ld_df(om, p0); K[4] = ld_df(ps, p0);
+      Kuv = fx::pair(ld_df(u, p0), ld_df(v, p0));
+      Kwp = fx::pair(ld_df(w, p0), ld_df(ps, p0));
+      Km = ld_df(om, p0);
     }
-    fx::acc s1[5], s2[7];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) s1[q].init(fx::df{0.f, 0.f});
-#pragma unroll
-    for (int q = 0; q < 7; ++q) s2[q].init(fx::df{0.f, 0.f});
+    // sums of the deviations (u, v), (w, psi) and of their products (uu, vv),
+    // (ww, psi psi), (uw, vw); (uv, the deviations of omega)
+    fx::acc2 suv, swp, quv, qwp, qw, qx;
+    {
+      const fx::df2 z{};
+      suv.init(z); swp.init(z); quv.init(z); qwp.init(z); qw.init(z); qx.init(z);
+    }
     // two particles per lane and iteration (positions i and i + 8), their
     // slots loaded one iteration ahead, so that ten state loads are in
     // flight before the first is needed; the sums still take the particles
@@ -524,19 +541,15 @@ __global__ void __launch_bounds__(256, 3) k_elem_stats_grp(const int32_t* __rest
     auto acc1 = [&](fx::df xu, fx::df xv, fx::df xw, fx::df xm, fx::df xp) {
       // normalized, so that the dropped product of the low parts is below
       // 2^-48 of the product even when the deviation is far below the value
-      const fx::df du = deviation(xu, K[0]);
-      const fx::df dv = deviation(xv, K[1]);
-      const fx::df dw = deviation(xw, K[2]);
-      const fx::df dm = deviation(xm, K[3]);
-      const fx::df dp = deviation(xp, K[4]);
-      s1[0].add(du); s1[1].add(dv); s1[2].add(dw); s1[3].add(dm); s1[4].add(dp);
-      s2[0].add(fx::mul(du, du));
-      s2[1].add(fx::mul(dv, dv));
-      s2[2].add(fx::mul(dw, dw));
-      s2[3].add(fx::mul(du, dv));
-      s2[4].add(fx::mul(du, dw));
-      s2[5].add(fx::mul(dv, dw));
-      s2[6].add(fx::mul(dp, dp));
+      const fx::df2 duv = deviation2(fx::pair(xu, xv), Kuv);
+      const fx::df2 dwp = deviation2(fx::pair(xw, xp), Kwp);
+      const fx::df dm = deviation(xm, Km);
+      suv.add(duv);
+      swp.add(dwp);
+      quv.add(fx::mul_df2(duv, duv));
+      qwp.add(fx::mul_df2(dwp, dwp));
+      qw.add(fx::mul_df2(duv, fx::pair(dwp.lane0(), dwp.lane0())));
+      qx.add(fx::pair(fx::mul(duv.lane0(), duv.lane1()), dm));
     };
     for (int32_t i = beg + j; i < end; i += 2 * kStatLanes) {
       const int32_t pa = qa, pb = qb;
@@ -552,11 +565,19 @@ __global__ void __launch_bounds__(256, 3) k_elem_stats_grp(const int32_t* __rest
     // butterfly within the group of eight: every lane ends with the totals
 #pragma unroll
     for (int o = kStatLanes / 2; o > 0; o >>= 1) {
-#pragma unroll
-      for (int q = 0; q < 5; ++q) acc_xor(s1[q], o);
-#pragma unroll
-      for (int q = 0; q < 7; ++q) acc_xor(s2[q], o);
+      acc_xor(suv, o);
+      acc_xor(swp, o);
+      acc_xor(quv, o);
+      acc_xor(qwp, o);
+      acc_xor(qw, o);
+      acc_xor(qx, o);
     }
+    auto one = [](float h, float l) { return fx::acc{h, l}; };
+    const fx::df K[5] = {Kuv.lane0(), Kuv.lane1(), Kwp.lane0(), Km, Kwp.lane1()};
+    const fx::acc s1[5] = {one(suv.h.x, suv.l.x), one(suv.h.y, suv.l.y), one(swp.h.x, swp.l.x), one(qx.h.y, qx.l.y),
+                           one(swp.h.y, swp.l.y)};
+    const fx::acc s2[7] = {one(quv.h.x, quv.l.x), one(quv.h.y, quv.l.y), one(qwp.h.x, qwp.l.x), one(qx.h.x, qx.l.x),
+                           one(qw.h.x, qw.l.x),   one(qw.h.y, qw.l.y),   one(qwp.h.y, qwp.l.y)};
     if (!live) continue;
     double* out = es + e * PDF_NES;
     if (N == 0) {

@@ -172,15 +172,23 @@ __device__ __forceinline__ void scale_row(const double a[PDF_NCOEF], const Coeff
 
 // The fixed-point kernel's row from the scaled FP64 row.
 __device__ __forceinline__ void make_fx_row(const double* r, FxRow* out) {
+  auto d = [&](int q) { return fx::d2df((uint64_t)__double_as_longlong(r[q])); };
   FxRow f;
-  const int mi[4] = {0, 1, 2, 26};
+  f.mean_uv = fx::pair(d(0), d(1));
+  f.mean_wp = fx::pair(d(2), d(26));
+  const fx::df sc = d(21);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) f.mean[j] = fx::d2df((uint64_t)__double_as_longlong(r[mi[j]]));
-  const int ci[23] = {3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16, 17, 18, 19, 20, 21, 23, 24, 25, 27};
-#pragma unroll
-  for (int q = 0; q < 23; ++q) f.c[q] = fx::d2df((uint64_t)__double_as_longlong(r[ci[q]]));
-#pragma unroll
-  for (int q = 23; q < 28; ++q) f.c[q] = fx::df{0.f, 0.f};
+  for (int i = 0; i < 3; ++i) {
+    f.grad[i] = fx::pair(d(3 + 2 * i), d(4 + 2 * i));
+    f.drift[i] = fx::pair(d(12 + 3 * i), d(13 + 3 * i));
+    f.rest[i] = fx::pair(d(14 + 3 * i), sc);
+    f.a[i] = d(9 + i);
+    f.pad[i] = fx::df{0.f, 0.f};
+  }
+  const fx::df c = d(23);
+  f.freq = fx::pair(fx::df{-c.h, -c.l}, d(25));
+  f.freq0 = d(24);
+  f.mix = d(27);
   *out = f;
 }
 
@@ -611,6 +619,15 @@ __global__ void __launch_bounds__(256) k_step(StepArgs A) {
 // product and sums by TwoSum.  A particle whose position increment
 // reaches one length unit, or whose walk meets a wall, an open boundary or
 // the step cap, is finished by the native FP64 code above.
+//
+// Instruction issue bounds it, with the FP32 pipe at a third of its rate: the
+// arithmetic runs two values per instruction (f2, df2 in fx.cuh) along pairs
+// that sit beside each other anyway: the two coordinates, the two Box-Muller
+// pairs of a block, and for each velocity component two sums side by side
+// whose products are formed from neighbouring coefficients, draws and
+// differences.  The row is laid out in those pairs (15 loads of 16 bytes
+// instead of 27 of 8).  15.9M particles: 914 -> 810 us; FP32 state (draws,
+// position and screen only), 5.1M particles: 245 -> 220 us.
 // ----------------------------------------------------------------------------
 constexpr int kF = kPosF;
 
@@ -618,8 +635,8 @@ struct FxArgs {
   const FxRow* rows;
   const FxGeo* geo;
   int64_t period_fix;
-  fx::df dt;      // dt
-  fx::df sdiff;   // sqrt(2 nu dt)
+  fx::df2 dt;      // dt, in both lanes
+  fx::df2 sdiff;   // sqrt(2 nu dt), in both lanes
   // concentrated source: 0 none, 1 double-float test with the FP64 test in
   // the rounding band, 2 FP64 test only (centre outside the fixed range)
   int src_mode;
@@ -627,13 +644,13 @@ struct FxArgs {
   fx::df src_r2;         // r^2
 };
 
-__device__ __forceinline__ fx::df ldc(const FxRow* r, int q) {
-  const float2 v = __ldg(reinterpret_cast<const float2*>(&r->c[q]));
-  return fx::df{v.x, v.y};
+__device__ __forceinline__ fx::df2 ld_pair(const fx::df2* a) {
+  const float4 v = __ldg(reinterpret_cast<const float4*>(a));
+  return fx::df2{fx::f2{v.x, v.y}, fx::f2{v.z, v.w}};
 }
 
-__device__ __forceinline__ fx::df ldmean(const FxRow* r, int j) {
-  const float2 v = __ldg(reinterpret_cast<const float2*>(&r->mean[j]));
+__device__ __forceinline__ fx::df ld_coef(const fx::df* a) {
+  const float2 v = __ldg(reinterpret_cast<const float2*>(a));
   return fx::df{v.x, v.y};
 }
 
@@ -644,15 +661,6 @@ __device__ __forceinline__ fx::df ld_state(const fx::df* a, int64_t p) {
 
 __device__ __forceinline__ void st_state(fx::df* a, int64_t p, fx::df v) {
   reinterpret_cast<float2*>(a)[p] = make_float2(v.h, v.l);
-}
-
-// a - b with the rounding error of the high parts kept (not renormalized;
-// used as a multiplicand).
-__device__ __forceinline__ fx::df dsub(fx::df a, fx::df b) {
-  fx::acc t;
-  t.init(a);
-  t.sub(b);
-  return fx::df{t.h, t.l};
 }
 
 // Twice the sub-areas in double-float (normalized), from fixed-point offsets.
@@ -685,8 +693,9 @@ struct Screen {
 
 __device__ __forceinline__ Screen screen_xy(int64_t xb, int64_t yb, float cbx, float cby, float abx, float aby,
                                             float two_area, int64_t X, int64_t Y) {
-  const fx::df dxd = fx::fix2df(X - xb, kF), dyd = fx::fix2df(Y - yb, kF);
-  const float dx = dxd.h + dxd.l, dy = dyd.h + dyd.l;
+  const fx::df2 d = fx::fix2df2(X - xb, Y - yb, kF);
+  const fx::f2 o = fx::add2(d.h, d.l);
+  const float dx = o.x, dy = o.y;
   const float p1 = cbx * dy, p2 = cby * dx;
   const float q1 = dx * aby, q2 = dy * abx;
   Screen S;
@@ -919,8 +928,12 @@ __device__ __forceinline__ bool in_source_fx(const StepArgs& A, const FxArgs& F,
 }
 
 // Position increment bound of the fixed-point path: |U dt + sqrt(2 nu dt) dW| < 1,
-// which keeps every fixed-point offset of the walk below 2^7.
-__device__ __forceinline__ bool small_move(const fx::acc& a) { return fabsf(a.h) < 1.0f; }
+// which keeps every fixed-point offset of the walk below 2^7, and low parts
+// within the fixed-point sum's range (they exceed it only where two large
+// terms cancel).
+__device__ __forceinline__ bool small_move(const fx::acc2& a) {
+  return fmaxf(fabsf(a.h.x), fabsf(a.h.y)) < 1.0f && fmaxf(fabsf(a.l.x), fabsf(a.l.y)) <= fx::kIncMax;
+}
 
 // FP64 back to the stored forms after the FP64 walk (the wall fall-back).
 __device__ __forceinline__ bool pos_fits(double x) { return fabs(x) < 64.0; }
@@ -959,69 +972,73 @@ __global__ void __launch_bounds__(256, 4) k_step_fx(StepArgs A, FxArgs F) {
     Draws D;
     const uint32_t id = (uint32_t)__ldg(A.pid + p);
     draw_block0(A, id, D);
-    const fx::df U[3] = {ld_state(A.u, p), ld_state(A.v, p), ld_state(A.w, p)};
-    // position (eq. Lagrangian-position-exact): X + U^n dt + sqrt(2 nu) dW
-    fx::acc ax, ay;
-    ax.init(fx::mul(U[0], F.dt));
-    ax.add(fx::mul_f(F.sdiff, D.g[0]));
-    ay.init(fx::mul(U[1], F.dt));
-    ay.add(fx::mul_f(F.sdiff, D.g[1]));
+    const fx::df2 Uuv = fx::pair(ld_state(A.u, p), ld_state(A.v, p));
+    const fx::df W = ld_state(A.w, p);
+    const fx::f2 g01 = {D.g[0], D.g[1]};
+    // position (eq. Lagrangian-position-exact): X + U^n dt + sqrt(2 nu) dW,
+    // the two coordinates lane by lane
+    fx::acc2 dxy;
+    dxy.init(fx::mul_df2(Uuv, F.dt));
+    dxy.add(fx::mul_f2(F.sdiff, g01));
     // large moves go to the FP64 path; so do particles next to a no-slip
     // wall (the flag is loaded here and tested after the SDE updates, so
     // that its latency is hidden)
     const int near_noslip = __ldg(reinterpret_cast<const int*>(F.geo + e) + 18);
-    if (!(small_move(ax) && small_move(ay))) {
+    if (!small_move(dxy)) {
       draw_block1(A, id, D);
       merge(cs, advance_native_ool(A, p, D));
       continue;
     }
-    int64_t Xn = A.x[p] + ax.fix(kF);
-    const int64_t Yn = A.y[p] + ay.fix(kF);
+    int64_t Xn = A.x[p], Yn = A.y[p];
+    fx::add_inc2(Xn, Yn, dxy.h, dxy.l);
     // the new position against the old element now, so that the geometry
     // of the neighbour it leaves into arrives during the SDE updates
     const int first = early_screen(F, e, Xn, Yn);
     draw_block1(A, id, D);
     // velocity prediction (eq. velocity-prediction): U + a dt
     // + sqrt(2 nu) dU_i/dx_j dW_j + G_ij (U_j - <U_j>) dt + sqrt(C0 eps) dW'_i
-    const fx::df d0 = dsub(U[0], ldmean(R, 0));
-    const fx::df d1 = dsub(U[1], ldmean(R, 1));
-    const fx::df d2 = dsub(U[2], ldmean(R, 2));
-    const fx::df sc = ldc(R, 18);
+    // Each row of three products by pairs is summed in two lanes, U_i and
+    // a_i dt starting one each: the pairs are what the row holds and what
+    // the draws and differences are, so nothing is moved between lanes.
+    const fx::df S = ld_state(A.ps, p);
+    fx::df2 mwp = ld_pair(&R->mean_wp);
+    if (A.cond) {  // IECM: the particle's velocity-conditioned mean <phi|V>
+      const fx::df cv = ld_state(A.cond, p);
+      mwp.h.y = cv.h;
+      mwp.l.y = cv.l;
+    }
+    const fx::df2 d01 = fx::dsub2(Uuv, ld_pair(&R->mean_uv));
+    const fx::df2 dwp = fx::dsub2(fx::pair(W, S), mwp);
+    const fx::df d2 = dwp.lane0();
     fx::df Un[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      fx::acc a;
-      a.init(U[i]);
-      a.add(ldc(R, 6 + i));
-      a.add(fx::mul_f(ldc(R, 2 * i), D.g[0]));
-      a.add(fx::mul_f(ldc(R, 2 * i + 1), D.g[1]));
-      a.add(fx::mul(ldc(R, 9 + 3 * i), d0));
-      a.add(fx::mul(ldc(R, 10 + 3 * i), d1));
-      a.add(fx::mul(ldc(R, 11 + 3 * i), d2));
-      a.add(fx::mul_f(sc, D.g[2 + i]));
-      Un[i] = a.value();
+      fx::acc2 a;
+      a.init(fx::pair(i == 0 ? Uuv.lane0() : (i == 1 ? Uuv.lane1() : W), ld_coef(&R->a[i])));
+      a.add(fx::mul_f2(ld_pair(&R->grad[i]), g01));
+      a.add(fx::mul_df2(ld_pair(&R->drift[i]), d01));
+      a.add(fx::mul_df2(ld_pair(&R->rest[i]), fx::pair(d2, fx::df{D.g[2 + i], 0.0f})));
+      Un[i] = a.fold().value();
     }
     // frequency (eq. frequency-model): omega - (C3 + S_w) <w> dt omega + C3 <w>^2 dt
     // + <w> sqrt(2 C3 C4 dt) sqrt(max(omega, 0)) dW
     const fx::df O = ld_state(A.om, p);
     fx::df On;
     {
-      fx::acc a;
-      a.init(O);
-      a.sub(fx::mul(ldc(R, 19), O));
-      a.add(ldc(R, 20));
-      a.add(fx::mul_f(fx::mul(ldc(R, 21), fx::sqrt_df(O)), D.g[5]));
-      On = a.value();
+      const fx::df2 f = fx::mul_df2(ld_pair(&R->freq), fx::pair(O, fx::sqrt_df(O)));
+      fx::acc2 a;
+      a.init(fx::pair(O, ld_coef(&R->freq0)));
+      a.add(fx::pair(f.lane0(), fx::mul_f(f.lane1(), D.g[5])));
+      On = a.fold().value();
       if (On.h < 0.0f) { On = fx::df{-On.h, -On.l}; ++c_om; }
     }
     // scalar: psi - (psi - <phi>) dt / t_m (eq. IEM) or with the particle's
     // velocity-conditioned mean <phi|V> (eq. IECM)
-    const fx::df S = ld_state(A.ps, p);
     fx::df Sn;
     {
       fx::acc a;
       a.init(S);
-      a.sub(fx::mul(ldc(R, 22), dsub(S, A.cond ? ld_state(A.cond, p) : ldmean(R, 3))));
+      a.sub(fx::mul(ld_coef(&R->mix), dwp.lane1()));
       Sn = a.value();
     }
     if (near_noslip) {
@@ -1135,18 +1152,14 @@ __global__ void __launch_bounds__(256, 4) k_step_f32(StepArgs A, FxArgs F, F32Ar
     }
     // position (eq. Lagrangian-position-exact), fixed point
     const int64_t X0 = A.x[p], Y0 = A.y[p];
-    fx::acc a;
-    a.init(fx::mul_f(F.dt, U0));
-    a.add(fx::mul_f(F.sdiff, D.g[0]));
-    fx::acc c;
-    c.init(fx::mul_f(F.dt, U1));
-    c.add(fx::mul_f(F.sdiff, D.g[1]));
+    fx::acc2 dxy;
+    dxy.init(fx::mul_f2(F.dt, fx::f2{U0, U1}));
+    dxy.add(fx::mul_f2(F.sdiff, fx::f2{D.g[0], D.g[1]}));
     int64_t Xn = X0, Yn = Y0;
     bool slow, reinj = false;
     double xn, yn;
-    if (small_move(a) && small_move(c)) {
-      Xn = X0 + a.fix(kF);
-      Yn = Y0 + c.fix(kF);
+    if (small_move(dxy)) {
+      fx::add_inc2(Xn, Yn, dxy.h, dxy.l);
       int steps = 0;
       slow = walk_fx(F, e, Xn, Yn, steps, c_per, c_near, reinj);
       c_walk += steps;
@@ -1345,9 +1358,9 @@ static StepLaunch step_args(pdf_particles* p, const pdf_mesh* m, const pdf_model
     std::memcpy(&b, &M.period, 8);
     F.period_fix = fx::d2fix(b, kF);
     std::memcpy(&b, &A.dt, 8);
-    F.dt = fx::d2df(b);
+    F.dt = fx::pair(fx::d2df(b), fx::d2df(b));
     std::memcpy(&b, &A.sdiff, 8);
-    F.sdiff = fx::d2df(b);
+    F.sdiff = fx::pair(fx::d2df(b), fx::d2df(b));
     F.src_mode = 0;
     F.src_x = F.src_y = 0;
     F.src_r2 = fx::df{0.f, 0.f};
