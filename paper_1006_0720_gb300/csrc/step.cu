@@ -1240,14 +1240,16 @@ static pdf_status check_params(const pdf_model_params* p) {
 }
 
 // Coefficient rows from the stored statistics (GLM/SLM).
+int pass_threads(int64_t n);  // stats.cu
+
 static pdf_status build_rows(pdf_particles* P, const pdf_model_params* params, const double* wp,
                              double* avg_out, bool internal, cudaStream_t st) {
   const MeshDev& M = P->mesh->d;
   const CoeffParams C = coeff_params(params);
-  PDF_KERNEL("k_node_coeff", st, k_node_coeff<<<blocks_for(M.n_nodes, 128, 32), 128, 0, st>>>(M.n_nodes, P->ns, P->nd,
+  PDF_KERNEL("k_node_coeff", st, k_node_coeff<<<blocks_for(M.n_nodes, pass_threads(M.n_nodes), 32), pass_threads(M.n_nodes), 0, st>>>(M.n_nodes, P->ns, P->nd,
                                                                 params->closure == PDF_CLOSURE_GLM ? wp : nullptr,
                                                                 M.xy, C, P->gradP, P->nc););
-  PDF_KERNEL("k_elem_rows", st, k_elem_rows<<<blocks_for(M.n_tri, 128, 32), 128, 0, st>>>(M.tri, M.n_tri, P->nc, C,
+  PDF_KERNEL("k_elem_rows", st, k_elem_rows<<<blocks_for(M.n_tri, pass_threads(M.n_tri), 32), pass_threads(M.n_tri), 0, st>>>(M.tri, M.n_tri, P->nc, C,
                                                              internal ? P->rows : nullptr, avg_out,
                                                              internal && C.arith == PDF_ARITH_FX ? P->rows_fx : nullptr,
                                                              internal ? P->rows_f32 : nullptr, M.geo, M.nsw_line,
@@ -1281,7 +1283,7 @@ static pdf_status step_prepare(pdf_particles* p, const pdf_mesh* m, const pdf_mo
   const MeshDev& M = m->d;
   if (params->closure == PDF_CLOSURE_FROZEN) {
     if (!elem_coeff) return fail(PDF_EINVAL, "pdf_step: FROZEN needs elem_coeff");
-    PDF_KERNEL("k_frozen_rows", st, k_frozen_rows<<<blocks_for(M.n_tri, 128, 32), 128, 0, st>>>(
+    PDF_KERNEL("k_frozen_rows", st, k_frozen_rows<<<blocks_for(M.n_tri, pass_threads(M.n_tri), 32), pass_threads(M.n_tri), 0, st>>>(
                                          M.n_tri, elem_coeff, coeff_params(params), p->rows,
                                          params->arith == PDF_ARITH_FX ? p->rows_fx : nullptr, p->rows_f32););
   } else {
