@@ -78,9 +78,10 @@ __device__ __forceinline__ int64_t scan_chunk(int64_t n_tiles, int64_t tile) {
   return (kScanChunks * (tile + 1) - 1) / n_tiles;
 }
 template <int BITS, int TILE>
-__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const int32_t* __restrict__ keys, int64_t n,
+__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const int32_t* keys, int64_t n,
                                                              int shift, int sub, int32_t* __restrict__ hist,
                                                              int32_t* __restrict__ sums) {
+  overlap_begin();
   constexpr int kBins = 1 << BITS, kPer = TILE / kSortThreads;
   __shared__ int32_t h[kBins];
   for (int b = threadIdx.x; b < kBins; b += kSortThreads) h[b] = 0;
@@ -92,12 +93,12 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const int32_t* __re
       const int4* q = reinterpret_cast<const int4*>(keys + i0);
 #pragma unroll
       for (int j = 0; j < kPer / 4; ++j) {
-        const int4 v = __ldg(q + j);
+        const int4 v = q[j];
         k[4 * j] = v.x; k[4 * j + 1] = v.y; k[4 * j + 2] = v.z; k[4 * j + 3] = v.w;
       }
     } else {
 #pragma unroll
-      for (int r = 0; r < kPer; ++r) k[r] = (i0 + r < n) ? __ldg(keys + i0 + r) : 0;
+      for (int r = 0; r < kPer; ++r) k[r] = (i0 + r < n) ? keys[i0 + r] : 0;
     }
     const int m = (int)max((int64_t)0, min((int64_t)kPer, n - i0));  // keys of this thread
     int run_d = -1, run_c = 0;
@@ -159,8 +160,9 @@ __device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t* tota
 // group of 32 digits (blockIdx.y), from the sums of the earlier chunks.
 // Thread (x, y) takes digit x of the group and the y-th of the chunk's eight
 // runs of tiles, so that a warp reads 128 consecutive bytes.
-__global__ void __launch_bounds__(256) k_scan_bins(int32_t* __restrict__ hist, int64_t n_tiles, int bins,
-                                                   const int32_t* __restrict__ sums, int32_t* __restrict__ part) {
+__global__ void __launch_bounds__(256) k_scan_bins(int32_t* hist, int64_t n_tiles, int bins,
+                                                   const int32_t* sums, int32_t* __restrict__ part) {
+  overlap_begin();
   __shared__ int32_t before[8][32], own[8][32];
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5, b = blockIdx.y * 32 + x;
   const int64_t c0 = n_tiles * blockIdx.x / kScanChunks, c1 = n_tiles * (blockIdx.x + 1) / kScanChunks;
@@ -168,7 +170,7 @@ __global__ void __launch_bounds__(256) k_scan_bins(int32_t* __restrict__ hist, i
   int32_t t = 0, p = 0;
 #pragma unroll
   for (int c = y; c < kScanChunks; c += 8) {  // the chunks before this one, and all
-    const int32_t v = __ldg(sums + c * bins + b);
+    const int32_t v = sums[c * bins + b];
     if (c < (int)blockIdx.x) p += v;
     t += v;
   }
@@ -217,9 +219,10 @@ constexpr size_t scatter_shared() {
 }
 template <int BITS, int TILE, bool FUSED>
 __global__ void __launch_bounds__(kScatterThreads, BITS <= 10 ? 2 : 1) k_radix_scatter(
-    const int32_t* __restrict__ keys_in, const int32_t* __restrict__ vals_in, int64_t n, int shift,
-    int sub, int64_t n_tiles, const int32_t* __restrict__ hist, int32_t* __restrict__ part,
+    const int32_t* keys_in, const int32_t* vals_in, int64_t n, int shift,
+    int sub, int64_t n_tiles, const int32_t* hist, int32_t* part,
     int32_t* __restrict__ keys_out, int32_t* __restrict__ vals_out, int32_t* __restrict__ seg, int32_t n_seg) {
+  overlap_begin();
   constexpr int kBins = 1 << BITS;
   constexpr int kWarps = kScatterThreads / 32;       // 16
   constexpr int kPerWarp = TILE / kWarps;            // 256 or 128 items
@@ -256,11 +259,11 @@ __global__ void __launch_bounds__(kScatterThreads, BITS <= 10 ? 2 : 1) k_radix_s
       int32_t c[kDig];
       const int32_t* h = hist + (int64_t)t * kBins + d0;
       if (kDig == 4) {
-        const int4 v = __ldg(reinterpret_cast<const int4*>(h));
+        const int4 v = *reinterpret_cast<const int4*>(h);
         c[0] = v.x; c[kDig - 3] = v.y; c[kDig - 2] = v.z; c[kDig - 1] = v.w;
       } else {
 #pragma unroll
-        for (int q = 0; q < kDig; ++q) c[q] = __ldg(h + q);
+        for (int q = 0; q < kDig; ++q) c[q] = h[q];
       }
 #pragma unroll
       for (int q = 0; q < kDig; ++q) {
@@ -285,7 +288,7 @@ __global__ void __launch_bounds__(kScatterThreads, BITS <= 10 ? 2 : 1) k_radix_s
   } else if (b0 < kBins) {
 #pragma unroll
     for (int q = 0; q < kDig; ++q) {
-      total[q] = __ldg(part + b0 + q);
+      total[q] = part[b0 + q];
       mine[q] = hist[(int64_t)blockIdx.x * kBins + b0 + q];
     }
     // the chunk sums behind part go back to zero for the next pass
@@ -370,23 +373,24 @@ __global__ void __launch_bounds__(kScatterThreads, BITS <= 10 ? 2 : 1) k_radix_s
 // per 16 positions, n / 16 + 1 threads in all.
 constexpr int kSegPer = 16;
 int64_t seg_offsets_threads(int64_t n) { return n / kSegPer + 1; }
-__global__ void __launch_bounds__(256) k_seg_offsets(const int32_t* __restrict__ keys, int64_t n, int32_t n_tri,
+__global__ void __launch_bounds__(256) k_seg_offsets(const int32_t* keys, int64_t n, int32_t n_tri,
                                                      int32_t* __restrict__ seg) {
+  overlap_begin();
   const int64_t i0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * kSegPer;
   int32_t k[kSegPer];
   if (i0 + kSegPer <= n && (reinterpret_cast<uintptr_t>(keys + i0) & 15) == 0) {
     const int4* q = reinterpret_cast<const int4*>(keys + i0);
 #pragma unroll
     for (int j = 0; j < kSegPer / 4; ++j) {
-      const int4 v = __ldg(q + j);
+      const int4 v = q[j];
       k[4 * j] = v.x; k[4 * j + 1] = v.y; k[4 * j + 2] = v.z; k[4 * j + 3] = v.w;
     }
   } else {
 #pragma unroll
-    for (int j = 0; j < kSegPer; ++j) k[j] = (i0 + j < n) ? __ldg(keys + i0 + j) : n_tri;
+    for (int j = 0; j < kSegPer; ++j) k[j] = (i0 + j < n) ? keys[i0 + j] : n_tri;
   }
   int32_t prev = __shfl_up_sync(0xffffffffu, k[kSegPer - 1], 1);
-  if ((threadIdx.x & 31) == 0) prev = (i0 == 0) ? -1 : ((i0 - 1 < n) ? __ldg(keys + i0 - 1) : n_tri);
+  if ((threadIdx.x & 31) == 0) prev = (i0 == 0) ? -1 : ((i0 - 1 < n) ? keys[i0 - 1] : n_tri);
   if (i0 > n) return;
 #pragma unroll
   for (int j = 0; j < kSegPer; ++j) {
@@ -496,11 +500,12 @@ __device__ __forceinline__ double moment(const fx::acc (&s1)[5], const fx::acc (
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256, 3) k_elem_stats_grp(const int32_t* __restrict__ seg,
+__global__ void __launch_bounds__(256, 3) k_elem_stats_grp(const int32_t* seg,
                                                        const int32_t* __restrict__ pid, int32_t n_tri,
                                                        const T* __restrict__ u, const T* __restrict__ v,
                                                        const T* __restrict__ w, const T* __restrict__ om,
                                                        const T* __restrict__ ps, double* __restrict__ es) {
+  overlap_begin();
   const int lane = threadIdx.x & 31, j = lane & (kStatLanes - 1);
   const int64_t group = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kStatLanes;
   const int64_t n_groups = ((int64_t)gridDim.x * blockDim.x) / kStatLanes;
@@ -630,8 +635,9 @@ __device__ __forceinline__ double recip_count(int32_t c) {
 // Node pass: mean over the non-empty surrounding elements (twins merged);
 // a node with none keeps its previous value.
 __global__ void k_node_stats(const int32_t* __restrict__ nse_off, const int32_t* __restrict__ nse,
-                             int32_t n_nodes, const double* __restrict__ es, double* __restrict__ ns,
+                             int32_t n_nodes, const double* es, double* ns,
                              long long* __restrict__ kept) {
+  overlap_begin();
   for (int32_t n = blockIdx.x * blockDim.x + threadIdx.x; n < n_nodes; n += gridDim.x * blockDim.x) {
     double acc[PDF_NNS];
 #pragma unroll
@@ -663,7 +669,8 @@ __global__ void k_node_stats(const int32_t* __restrict__ nse_off, const int32_t*
 // Element gradients of nodal <U>, <V>, <W>, <vv> (eq. gradient with the
 // analytic shape-function derivatives): eg[e] = Ux Uy Vx Vy Wx Wy vvx vvy.
 __global__ void k_elem_grad1(const int32_t* __restrict__ tri, const double* __restrict__ dN,
-                             int32_t n_tri, const double* __restrict__ ns, double* __restrict__ eg) {
+                             int32_t n_tri, const double* ns, double* __restrict__ eg) {
+  overlap_begin();
   for (int32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n_tri; e += gridDim.x * blockDim.x) {
     const double* d = dN + (int64_t)e * 6;
     double g[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -683,7 +690,8 @@ __global__ void k_elem_grad1(const int32_t* __restrict__ tri, const double* __re
 }
 
 __global__ void k_node_grad1(const int32_t* __restrict__ nse_off, const int32_t* __restrict__ nse,
-                             int32_t n_nodes, const double* __restrict__ eg, double* __restrict__ nd) {
+                             int32_t n_nodes, const double* eg, double* __restrict__ nd) {
+  overlap_begin();
   for (int32_t n = blockIdx.x * blockDim.x + threadIdx.x; n < n_nodes; n += gridDim.x * blockDim.x) {
     double acc[7] = {0, 0, 0, 0, 0, 0, 0};
     const int32_t b = nse_off[n], c = nse_off[n + 1] - b;
@@ -703,7 +711,8 @@ __global__ void k_node_grad1(const int32_t* __restrict__ nse_off, const int32_t*
 
 // Second pass: d/dx of the node dU_i/dx plus d/dy of the node dU_i/dy.
 __global__ void k_elem_grad2(const int32_t* __restrict__ tri, const double* __restrict__ dN,
-                             int32_t n_tri, const double* __restrict__ nd, double* __restrict__ eg) {
+                             int32_t n_tri, const double* nd, double* __restrict__ eg) {
+  overlap_begin();
   for (int32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n_tri; e += gridDim.x * blockDim.x) {
     const double* d = dN + (int64_t)e * 6;
     double l[3] = {0, 0, 0};
@@ -719,7 +728,8 @@ __global__ void k_elem_grad2(const int32_t* __restrict__ tri, const double* __re
 }
 
 __global__ void k_node_grad2(const int32_t* __restrict__ nse_off, const int32_t* __restrict__ nse,
-                             int32_t n_nodes, const double* __restrict__ eg, double* __restrict__ nd) {
+                             int32_t n_nodes, const double* eg, double* __restrict__ nd) {
+  overlap_begin();
   for (int32_t n = blockIdx.x * blockDim.x + threadIdx.x; n < n_nodes; n += gridDim.x * blockDim.x) {
     double acc[3] = {0, 0, 0};
     const int32_t b = nse_off[n], c = nse_off[n + 1] - b;
@@ -759,6 +769,11 @@ int pass_threads(int64_t n) {
   while (t > 32 && (n + t - 1) / t < 4 * (int64_t)sm_count()) t /= 2;
   return t;
 }
+int pass_blocks(int64_t n) { return blocks_for(n, pass_threads(n)); }
+
+// Whether a pass over n nodes or elements overlaps its predecessor (see
+// launch_over): blocks of one warp, at most two or three on an SM.
+static bool small_pass(int64_t n) { return pass_threads(n) == 32; }
 
 // One stable pass of the radix sort on the digit at `shift` (see RadixPlan).
 template <int BITS, int TILE, bool FUSED>
@@ -772,11 +787,13 @@ static pdf_status radix_pass_t(const RadixPlan& R, const int32_t* kin, const int
                                   (int)bytes));
   constexpr int kBins = 1 << BITS;
   int32_t* sums = FUSED ? nullptr : part + kBins;
-  PDF_KERNEL("k_radix_hist", st, k_radix_hist<BITS, TILE><<<nt, kSortThreads, 0, st>>>(kin, n, shift, R.sub, hist, sums););
+  PDF_KERNEL("k_radix_hist", st, launch_over(overlap(n), k_radix_hist<BITS, TILE>, nt, kSortThreads, 0, st, kin, n, shift,
+             R.sub, hist, sums););
   if (!FUSED)
-    PDF_KERNEL("k_scan_bins", st, k_scan_bins<<<dim3(kScanChunks, kBins / 32), 256, 0, st>>>(hist, R.tiles, kBins, sums, part););
-  PDF_KERNEL("k_radix_scatter", st, k_radix_scatter<BITS, TILE, FUSED><<<nt, kScatterThreads, bytes, st>>>(
-                                        kin, vin, n, shift, R.sub, R.tiles, hist, part, kout, vout, seg, n_seg););
+    PDF_KERNEL("k_scan_bins", st, launch_over(overlap(n), k_scan_bins, dim3(kScanChunks, kBins / 32), 256, 0, st, hist,
+               R.tiles, kBins, sums, part););
+  PDF_KERNEL("k_radix_scatter", st, launch_over(overlap(n), k_radix_scatter<BITS, TILE, FUSED>, nt, kScatterThreads, bytes,
+             st, kin, vin, n, shift, R.sub, R.tiles, hist, part, kout, vout, seg, n_seg););
   return PDF_OK;
 }
 template <int BITS>
@@ -818,8 +835,8 @@ static pdf_status group_keys(const RadixPlan& R, const int32_t* elem, int64_t n,
     vin = vout[pass];
   }
   if (!one)
-    PDF_KERNEL("k_seg_offsets", st, k_seg_offsets<<<(unsigned)((seg_offsets_threads(n) + 255) / 256), 256, 0, st>>>(
-                                        kin, n, n_tri, seg););
+    PDF_KERNEL("k_seg_offsets", st, launch_over(overlap(n), k_seg_offsets,
+               (unsigned)((seg_offsets_threads(n) + 255) / 256), 256, 0, st, kin, n, n_tri, seg););
   return PDF_OK;
 }
 
@@ -849,6 +866,7 @@ struct ReorderArgs {
 };
 
 __global__ void k_reorder(ReorderArgs R) {
+  overlap_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < R.n; i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t j = R.idx[i];
 #pragma unroll
@@ -885,7 +903,7 @@ static pdf_status launch_reorder(pdf_particles* P, cudaStream_t st) {
   add4(P->pid, P->pid2);
   // one thread per particle (0.31 ms at 15.9M particles against 0.46 ms
   // for a grid of 32 blocks per SM striding over them)
-  PDF_KERNEL("k_reorder", st, k_reorder<<<(unsigned)((P->n + 255) / 256), 256, 0, st>>>(R););
+  PDF_KERNEL("k_reorder", st, launch_over(overlap(P->n), k_reorder, (unsigned)((P->n + 255) / 256), 256, 0, st, R););
   return PDF_OK;
 }
 
@@ -917,11 +935,11 @@ static pdf_status elem_stats(pdf_particles* P, const int32_t* seg, const int32_t
   const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)M.n_tri * kStatLanes + 255) / 256,
                                                            (int64_t)sm_count() * 48));
   if (P->precision == PDF_FP64)
-    PDF_KERNEL("k_elem_stats", st, k_elem_stats_grp<fx::df><<<nb, 256, 0, st>>>(
-                                       seg, order, M.n_tri, P->u, P->v, P->w, P->om, P->ps, P->es));
+    PDF_KERNEL("k_elem_stats", st, launch_over(overlap(P->n), k_elem_stats_grp<fx::df>, nb, 256, 0, st, seg, order, M.n_tri,
+               P->u, P->v, P->w, P->om, P->ps, P->es));
   else
-    PDF_KERNEL("k_elem_stats", st, k_elem_stats_grp<float><<<nb, 256, 0, st>>>(
-                                       seg, order, M.n_tri, P->uf, P->vf, P->wf, P->omf, P->psf, P->es));
+    PDF_KERNEL("k_elem_stats", st, launch_over(overlap(P->n), k_elem_stats_grp<float>, nb, 256, 0, st, seg, order, M.n_tri,
+               P->uf, P->vf, P->wf, P->omf, P->psf, P->es));
   return PDF_OK;
 }
 
@@ -931,17 +949,21 @@ static pdf_status elem_stats(pdf_particles* P, const int32_t* seg, const int32_t
 // (sec. 3.3 second pass, sec. 3.4).
 pdf_status node_stats_from_elements(pdf_particles* P, cudaStream_t st) {
   const MeshDev& M = P->mesh->d;
-  PDF_KERNEL("k_node_stats", st, k_node_stats<<<blocks_for(M.n_nodes, pass_threads(M.n_nodes)), pass_threads(M.n_nodes), 0, st>>>(M.nse_off, M.nse, M.n_nodes, P->es, P->ns,
-                                                          P->counters + 8););
+  PDF_KERNEL("k_node_stats", st, launch_over(small_pass(M.n_nodes), k_node_stats, pass_blocks(M.n_nodes),
+             pass_threads(M.n_nodes), 0, st, M.nse_off, M.nse, M.n_nodes, P->es, P->ns, P->counters + 8););
   return node_derivs_from_node_stats(P, st);
 }
 
 pdf_status node_derivs_from_node_stats(pdf_particles* P, cudaStream_t st) {
   const MeshDev& M = P->mesh->d;
-  PDF_KERNEL("k_elem_grad1", st, k_elem_grad1<<<blocks_for(M.n_tri, pass_threads(M.n_tri)), pass_threads(M.n_tri), 0, st>>>(M.tri, M.dN, M.n_tri, P->ns, P->eg););
-  PDF_KERNEL("k_node_grad1", st, k_node_grad1<<<blocks_for(M.n_nodes, pass_threads(M.n_nodes)), pass_threads(M.n_nodes), 0, st>>>(M.nse_off, M.nse, M.n_nodes, P->eg, P->nd););
-  PDF_KERNEL("k_elem_grad2", st, k_elem_grad2<<<blocks_for(M.n_tri, pass_threads(M.n_tri)), pass_threads(M.n_tri), 0, st>>>(M.tri, M.dN, M.n_tri, P->nd, P->eg););
-  PDF_KERNEL("k_node_grad2", st, k_node_grad2<<<blocks_for(M.n_nodes, pass_threads(M.n_nodes)), pass_threads(M.n_nodes), 0, st>>>(M.nse_off, M.nse, M.n_nodes, P->eg, P->nd););
+  PDF_KERNEL("k_elem_grad1", st, launch_over(small_pass(M.n_tri), k_elem_grad1, pass_blocks(M.n_tri),
+             pass_threads(M.n_tri), 0, st, M.tri, M.dN, M.n_tri, P->ns, P->eg););
+  PDF_KERNEL("k_node_grad1", st, launch_over(small_pass(M.n_nodes), k_node_grad1, pass_blocks(M.n_nodes),
+             pass_threads(M.n_nodes), 0, st, M.nse_off, M.nse, M.n_nodes, P->eg, P->nd););
+  PDF_KERNEL("k_elem_grad2", st, launch_over(small_pass(M.n_tri), k_elem_grad2, pass_blocks(M.n_tri),
+             pass_threads(M.n_tri), 0, st, M.tri, M.dN, M.n_tri, P->nd, P->eg););
+  PDF_KERNEL("k_node_grad2", st, launch_over(small_pass(M.n_nodes), k_node_grad2, pass_blocks(M.n_nodes),
+             pass_threads(M.n_nodes), 0, st, M.nse_off, M.nse, M.n_nodes, P->eg, P->nd););
   return PDF_OK;
 }
 

@@ -88,9 +88,10 @@ __device__ void relax_rhs(const double* S, const double* D, const CoeffParams& P
 // <U_i>; d<U_i>/dx_j; a_i = -d<P>/dx_i + 2 nu lap<U_i> (GLM) or -d<P>/dx_i
 // (SLM); G_ij (eq. GandC or eq. wall-GandC); sqrt(C0 eps); <omega>; S_omega
 // (eq. frequency-source); <phi>; 1/t_m.
-__global__ void k_node_coeff(int32_t n_nodes, const double* __restrict__ ns, const double* __restrict__ nd,
-                             const double* __restrict__ wp, const double* __restrict__ xy, CoeffParams P,
-                             const double* __restrict__ gradP, double* __restrict__ nc) {
+__global__ void k_node_coeff(int32_t n_nodes, const double* ns, const double* nd,
+                             const double* wp, const double* __restrict__ xy, CoeffParams P,
+                             const double* gradP, double* __restrict__ nc) {
+  overlap_begin();
   for (int32_t n = blockIdx.x * blockDim.x + threadIdx.x; n < n_nodes; n += gridDim.x * blockDim.x) {
     double S[PDF_NNS], D[PDF_NND];
     for (int q = 0; q < PDF_NNS; ++q) S[q] = ns[(int64_t)n * PDF_NNS + q];
@@ -210,11 +211,12 @@ __device__ __forceinline__ double noslip_omega(int32_t e, const int32_t* tri, co
   return w > 0.0 ? w : om / 3.0;
 }
 
-__global__ void k_elem_rows(const int32_t* __restrict__ tri, int32_t n_tri, const double* __restrict__ nc,
+__global__ void k_elem_rows(const int32_t* __restrict__ tri, int32_t n_tri, const double* nc,
                             CoeffParams P, double* __restrict__ rows, double* __restrict__ avg_out,
                             FxRow* __restrict__ rows_fx, float* __restrict__ rows_f32,
                             const ElemGeo* __restrict__ geo, const double* __restrict__ nsw_line,
-                            const double* __restrict__ ns, const double* __restrict__ dN) {
+                            const double* ns, const double* __restrict__ dN) {
+  overlap_begin();
   for (int32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n_tri; e += gridDim.x * blockDim.x) {
     // node rows of 26 doubles (208 B, 16-byte aligned): 16-byte loads, and
     // 16-byte stores of the 256-byte element row (the kernel's loads and
@@ -225,7 +227,7 @@ __global__ void k_elem_rows(const int32_t* __restrict__ tri, int32_t n_tri, cons
     double a[PDF_NCOEF];
 #pragma unroll
     for (int q = 0; q < PDF_NCOEF / 2; ++q) {
-      const double2 x0 = __ldg(c0 + q), x1 = __ldg(c1 + q), x2 = __ldg(c2 + q);
+      const double2 x0 = c0[q], x1 = c1[q], x2 = c2[q];
       a[2 * q] = (x0.x + x1.x + x2.x) * (1.0 / 3.0);
       a[2 * q + 1] = (x0.y + x1.y + x2.y) * (1.0 / 3.0);
     }
@@ -248,8 +250,9 @@ __global__ void k_elem_rows(const int32_t* __restrict__ tri, int32_t n_tri, cons
   }
 }
 
-__global__ void k_frozen_rows(int32_t n_tri, const double* __restrict__ coeff, CoeffParams P,
+__global__ void k_frozen_rows(int32_t n_tri, const double* coeff, CoeffParams P,
                               double* __restrict__ rows, FxRow* __restrict__ rows_fx, float* __restrict__ rows_f32) {
+  overlap_begin();
   for (int32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < n_tri; e += gridDim.x * blockDim.x) {
     double a[PDF_NCOEF];
     for (int q = 0; q < PDF_NCOEF; ++q) a[q] = coeff[(int64_t)e * PDF_NCOEF + q];
@@ -455,7 +458,7 @@ __device__ __forceinline__ void draw_block1(const StepArgs& A, uint32_t id, Draw
 
 __device__ __forceinline__ Draws draw_step(const StepArgs& A, int64_t slot) {
   Draws d;
-  const uint32_t id = (uint32_t)__ldg(A.pid + slot);
+  const uint32_t id = (uint32_t)A.pid[slot];
   draw_block0(A, id, d);
   draw_block1(A, id, d);
   return d;
@@ -600,6 +603,7 @@ __device__ __forceinline__ void flush_counts(const StepArgs& A, const Counts& c)
 }
 
 __global__ void __launch_bounds__(256) k_step(StepArgs A) {
+  overlap_begin();
   Counts c;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   // every lane runs the same number of iterations so the warp reductions below see all lanes
@@ -942,6 +946,7 @@ __device__ __forceinline__ bool pos_fits(double x) { return fabs(x) < 64.0; }
 
 __global__ void __launch_bounds__(256, 4) k_step_fx(const __grid_constant__ StepArgs A,
                                                     const __grid_constant__ FxArgs F) {
+  overlap_begin();
   int c_walk = 0, c_per = 0, c_om = 0, c_near = 0;
   Counts cs;  // counts of the FP64 fall-backs
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -972,7 +977,7 @@ __global__ void __launch_bounds__(256, 4) k_step_fx(const __grid_constant__ Step
     // the first random block (dW_x, dW_y, dW'_1, dW'_2) gives the position;
     // the second is drawn after the early screen below
     Draws D;
-    const uint32_t id = (uint32_t)__ldg(A.pid + p);
+    const uint32_t id = (uint32_t)A.pid[p];
     draw_block0(A, id, D);
     const fx::df2 Uuv = fx::pair(ld_state(A.u, p), ld_state(A.v, p));
     const fx::df W = ld_state(A.w, p);
@@ -1238,6 +1243,7 @@ template <bool QUEUE>
 __global__ void __launch_bounds__(kStepThreads, 4) k_step_f32(const __grid_constant__ StepArgs A,
                                                               const __grid_constant__ FxArgs F,
                                                               const __grid_constant__ F32Args S) {
+  overlap_begin();
   __shared__ WalkQueue<QUEUE ? kQueue : 1> queues[kStepThreads / 32];
   auto& Q = queues[threadIdx.x >> 5];
   int queued = 0;
@@ -1360,19 +1366,19 @@ static pdf_status check_params(const pdf_model_params* p) {
 
 // Coefficient rows from the stored statistics (GLM/SLM).
 int pass_threads(int64_t n);  // stats.cu
+int pass_blocks(int64_t n);
 
 static pdf_status build_rows(pdf_particles* P, const pdf_model_params* params, const double* wp,
                              double* avg_out, bool internal, cudaStream_t st) {
   const MeshDev& M = P->mesh->d;
   const CoeffParams C = coeff_params(params);
-  PDF_KERNEL("k_node_coeff", st, k_node_coeff<<<blocks_for(M.n_nodes, pass_threads(M.n_nodes), 32), pass_threads(M.n_nodes), 0, st>>>(M.n_nodes, P->ns, P->nd,
-                                                                params->closure == PDF_CLOSURE_GLM ? wp : nullptr,
-                                                                M.xy, C, P->gradP, P->nc););
-  PDF_KERNEL("k_elem_rows", st, k_elem_rows<<<blocks_for(M.n_tri, pass_threads(M.n_tri), 32), pass_threads(M.n_tri), 0, st>>>(M.tri, M.n_tri, P->nc, C,
-                                                             internal ? P->rows : nullptr, avg_out,
-                                                             internal && C.arith == PDF_ARITH_FX ? P->rows_fx : nullptr,
-                                                             internal ? P->rows_f32 : nullptr, M.geo, M.nsw_line,
-                                                             P->ns, M.dN););
+  PDF_KERNEL("k_node_coeff", st, launch_over(overlap(P->n), k_node_coeff, pass_blocks(M.n_nodes), pass_threads(M.n_nodes), 0,
+             st, M.n_nodes, P->ns, P->nd, params->closure == PDF_CLOSURE_GLM ? wp : nullptr, M.xy, C, P->gradP,
+             P->nc););
+  PDF_KERNEL("k_elem_rows", st, launch_over(overlap(P->n), k_elem_rows, pass_blocks(M.n_tri), pass_threads(M.n_tri), 0, st,
+             M.tri, M.n_tri, P->nc, C, internal ? P->rows : nullptr, avg_out,
+             internal && C.arith == PDF_ARITH_FX ? P->rows_fx : nullptr, internal ? P->rows_f32 : nullptr, M.geo,
+             M.nsw_line, P->ns, M.dN););
   return PDF_OK;
 }
 
@@ -1402,9 +1408,9 @@ static pdf_status step_prepare(pdf_particles* p, const pdf_mesh* m, const pdf_mo
   const MeshDev& M = m->d;
   if (params->closure == PDF_CLOSURE_FROZEN) {
     if (!elem_coeff) return fail(PDF_EINVAL, "pdf_step: FROZEN needs elem_coeff");
-    PDF_KERNEL("k_frozen_rows", st, k_frozen_rows<<<blocks_for(M.n_tri, pass_threads(M.n_tri), 32), pass_threads(M.n_tri), 0, st>>>(
-                                         M.n_tri, elem_coeff, coeff_params(params), p->rows,
-                                         params->arith == PDF_ARITH_FX ? p->rows_fx : nullptr, p->rows_f32););
+    PDF_KERNEL("k_frozen_rows", st, launch_over(overlap(p->n), k_frozen_rows, pass_blocks(M.n_tri), pass_threads(M.n_tri), 0,
+               st, M.n_tri, elem_coeff, coeff_params(params), p->rows,
+               params->arith == PDF_ARITH_FX ? p->rows_fx : nullptr, p->rows_f32););
   } else {
     if (!p->have_stats) return fail(PDF_ESTATE, "pdf_step: call pdf_estimate_stats before a GLM/SLM step");
     s = build_rows(p, params, wp, nullptr, true, st);
@@ -1429,6 +1435,7 @@ struct StepLaunch {
   pdf_status run(int64_t beg, int64_t cnt, cudaStream_t st, int per_sm = 16) const {
     if (cnt <= 0) return PDF_OK;
     const int nb = blocks_for(cnt, 256, per_sm);
+    const bool over = cnt <= kOverlapStepMax;
     StepArgs a = A;
     a.n = cnt;
     a.x += beg; a.y += beg; a.elem += beg; a.pid += beg;
@@ -1439,15 +1446,15 @@ struct StepLaunch {
       // the queue where a warp takes eight rounds or more and fills it; with
       // fewer the last, partial one is a longer chain than the walk itself
       if (cnt >= 8 * (int64_t)nb * kStepThreads)
-        PDF_KERNEL("k_step", st, k_step_f32<true><<<nb, kStepThreads, 0, st>>>(a, F, f));
+        PDF_KERNEL("k_step", st, launch_over(over, k_step_f32<true>, nb, kStepThreads, 0, st, a, F, f));
       else
-        PDF_KERNEL("k_step", st, k_step_f32<false><<<nb, kStepThreads, 0, st>>>(a, F, f));
+        PDF_KERNEL("k_step", st, launch_over(over, k_step_f32<false>, nb, kStepThreads, 0, st, a, F, f));
     } else if (kind == 1) {
       a.u += beg; a.v += beg; a.w += beg; a.om += beg; a.ps += beg;
-      PDF_KERNEL("k_step", st, k_step_fx<<<nb, 256, 0, st>>>(a, F));
+      PDF_KERNEL("k_step", st, launch_over(over, k_step_fx, nb, 256, 0, st, a, F));
     } else {
       a.u += beg; a.v += beg; a.w += beg; a.om += beg; a.ps += beg;
-      PDF_KERNEL("k_step", st, k_step<<<nb, 256, 0, st>>>(a));
+      PDF_KERNEL("k_step", st, launch_over(over, k_step, nb, 256, 0, st, a));
     }
     return PDF_OK;
   }
