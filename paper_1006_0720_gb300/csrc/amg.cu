@@ -69,17 +69,19 @@ HCsr transpose(const HCsr& A) {
   return T;  // columns ascending within each row
 }
 
-// f(lo, hi, chunk) over chunks of the rows [0, n) on several host threads (the
-// set-up runs at the first solve of a mesh, on its critical path).  Throws
-// std::bad_alloc when a chunk did.
+// f(lo, hi, chunk) over chunks of at least `grain` of the rows [0, n) on
+// several host threads (the set-up runs at the first solve of a mesh, on its
+// critical path).  A thread costs some 30 us to start: chunks of a matrix
+// product or a plan (about a microsecond a row) from 512 rows, of a power
+// iteration (20 ns a row) from 8,192.  Throws std::bad_alloc when a chunk did.
 constexpr int kMaxChunks = 16;
-int row_chunks(int32_t n) {
+int row_chunks(int32_t n, int32_t grain) {
   const int hw = (int)std::thread::hardware_concurrency();
-  return std::max(1, std::min({kMaxChunks, hw > 0 ? hw : 1, n / 1024}));
+  return std::max(1, std::min({kMaxChunks, hw > 0 ? hw : 1, n / grain}));
 }
 template <typename F>
-void parallel_rows(int32_t n, F f) {
-  const int c = row_chunks(n);
+void parallel_rows(int32_t n, F f, int32_t grain = 512) {
+  const int c = row_chunks(n, grain);
   std::atomic<bool> failed{false};
   auto run = [&](int k) {
     try {
@@ -231,7 +233,7 @@ double eigen_bound(const HCsr& A, const std::vector<double>& d) {
       }
       sum[k] = s2;
       gersh[k] = g;
-    });
+    }, 8192);
     double t = 0.0;
     for (double s : sum) t += s;
     if (!(t > 0.0)) break;
@@ -915,14 +917,15 @@ void relax_amg_free(RelaxAmg& G) {
     cudaFree(L.s_rp); cudaFree(L.s_ci); cudaFree(L.s_perm); cudaFree(L.ap_off); cudaFree(L.ap_qa);
     cudaFree(L.ap_pv); cudaFree(L.c_off); cudaFree(L.c_tap); cudaFree(L.c_pv); cudaFree(L.q_pin);
     cudaFree(L.q_row); cudaFree(L.b); cudaFree(L.x); cudaFree(L.z);
+    cudaFree(L.ap_v);
     for (int v = 0; v < kRxVar; ++v) {
-      cudaFree(L.a_v[v]); cudaFree(L.ap_v[v]); cudaFree(L.q_v[v]); cudaFree(L.s_v[v]);
+      cudaFree(L.a_v[v]);
       cudaFree(L.a_f[v]); cudaFree(L.q_f[v]); cudaFree(L.s_f[v]); cudaFree(L.w_f[v]); cudaFree(L.w_v[v]);
     }
   }
   cudaFree(G.c_rp); cudaFree(G.c_ci);
   for (int v = 0; v < kRxVar; ++v) cudaFree(G.c_v[v]);
-  cudaFree(G.cmat); cudaFree(G.cinv); cudaFree(G.r32); cudaFree(G.omega); cudaFree(G.gpart);
+  cudaFree(G.cinv); cudaFree(G.r32); cudaFree(G.omega); cudaFree(G.gpart);
   cudaFree(G.upart);
   G = RelaxAmg();
 }
@@ -992,6 +995,7 @@ static pdf_status relax_amg_setup_host(int32_t n, const std::vector<int32_t>& rp
       }
     }
     L.nnz_ap = nap;
+    L.ap_terms = (int64_t)ap.id.size();
     // S = Q^T with the permutation of the entries
     std::vector<int32_t> s_rp(P.m + 1, 0), s_ci(nap), s_perm(nap);
     for (int64_t t = 0; t < nap; ++t) s_rp[q_ci[t] + 1]++;
@@ -1013,6 +1017,7 @@ static pdf_status relax_amg_setup_host(int32_t n, const std::vector<int32_t>& rp
         for (int32_t t = q_rp[i]; t < q_rp[i + 1]; ++t) add(q_ci[t], t, Pt.v[k]);
       }
     });
+    L.c_terms = (int64_t)nx.id.size();
     if ((s = up_vec(&L.a_rp, a_rp)) != PDF_OK || (s = up_vec(&L.a_ci, a_ci)) != PDF_OK ||
         (s = up_vec(&L.a_dpos, dpos)) != PDF_OK || (s = up_vec(&L.q_rp, q_rp)) != PDF_OK ||
         (s = up_vec(&L.q_ci, q_ci)) != PDF_OK || (s = up_vec(&L.s_rp, s_rp)) != PDF_OK ||
@@ -1022,9 +1027,9 @@ static pdf_status relax_amg_setup_host(int32_t n, const std::vector<int32_t>& rp
         (s = up_vec(&L.c_tap, nx.id)) != PDF_OK || (s = up_vec(&L.c_pv, nx.w)) != PDF_OK ||
         (s = up_vec(&L.q_pin, q_pin)) != PDF_OK || (s = up_vec(&L.q_row, q_row)) != PDF_OK)
       break;
+    if ((s = zeros(&L.ap_v, kRxVar * nap)) != PDF_OK) break;
     for (int v = 0; v < kRxVar && s == PDF_OK; ++v)
-      if ((s = zeros(&L.a_v[v], L.nnz_a)) != PDF_OK || (s = zeros(&L.ap_v[v], nap)) != PDF_OK ||
-          (s = zeros(&L.q_v[v], nap)) != PDF_OK || (s = zeros(&L.s_v[v], nap)) != PDF_OK ||
+      if ((s = zeros(&L.a_v[v], L.nnz_a)) != PDF_OK ||
           (s = zeros(&L.a_f[v], L.nnz_a)) != PDF_OK || (s = zeros(&L.q_f[v], nap)) != PDF_OK ||
           (s = zeros(&L.s_f[v], nap)) != PDF_OK || (s = zeros(&L.w_f[v], (int64_t)na)) != PDF_OK ||
           (s = zeros(&L.w_v[v], (int64_t)na)) != PDF_OK)
@@ -1046,7 +1051,6 @@ static pdf_status relax_amg_setup_host(int32_t n, const std::vector<int32_t>& rp
     s = up_vec(&G.c_rp, a_rp);
     if (s == PDF_OK) s = up_vec(&G.c_ci, a_ci);
     for (int v = 0; v < kRxVar && s == PDF_OK; ++v) s = zeros(&G.c_v[v], G.nnz_c);
-    if (s == PDF_OK) s = zeros(&G.cmat, (int64_t)kRxVar * na * 2 * na);
     if (s == PDF_OK) s = zeros(&G.cinv, (int64_t)kRxVar * na * na);
     if (s == PDF_OK) s = zeros(&G.r32, 9 * (int64_t)n);
     if (s == PDF_OK) s = zeros(&G.omega, kRxVar * kRxMaxLv);
@@ -1061,28 +1065,61 @@ static pdf_status relax_amg_setup_host(int32_t n, const std::vector<int32_t>& rp
 // Per-variant pointers of one level, for the kernels.
 struct RxVals {
   const double* a[kRxVar];
-  double* ap[kRxVar];
-  double* q[kRxVar];
-  double* s[kRxVar];
+  double4_32a* ap;         // A P, the four variants of an entry side by side
   double* an[kRxVar];  // the next level's matrix values
   float *af[kRxVar], *qf[kRxVar], *sf[kRxVar], *wf[kRxVar];
   double* w[kRxVar];
 };
 
 // (A P)[t] for the four variants (each thread all four: the plan's indices
-// are loaded once).
-__global__ void k_rx_ap(int64_t nnz_ap, const int32_t* __restrict__ off, const int32_t* __restrict__ qa,
-                        const double* __restrict__ pv, RxVals V) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nnz_ap; t += (int64_t)gridDim.x * blockDim.x) {
+// are loaded once).  The four values of an entry are stored side by side:
+// k_rx_next gathers them, and from four arrays each gather moved four sectors
+// of 32 bytes for 32 bytes used.  G lanes per entry (the group's own part of
+// the terms, then a butterfly): one thread per entry was a chain of dependent
+// loads, up to hundreds of terms long on the coarsest levels, with few blocks.
+// 79,600 unknowns, four levels: k_rx_ap 355 -> 336 us, k_rx_next 403 -> 283 us
+// (eight lanes everywhere 402 and 372: the FP64 sums across the lanes); 760
+// unknowns, three levels: 55 -> 27 and 66 -> 25 us.
+// Entries from which one thread each is enough, and mean terms above which an
+// entry takes a warp.
+constexpr int64_t kRxThreads = 65536, kRxMany = 64;
+// The G lanes' sums of four values; lanes 0 to 3 end with one value each, of
+// variant rx_variant.  (Each stage halves the values a lane carries: four FP64
+// additions a lane where a butterfly of all four takes twelve.)
+template <int G>
+__device__ __forceinline__ double rx_group_sum(const double s[kRxVar]) {
+  static_assert(kRxVar == 4, "four variants");
+  const uint32_t m = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << (threadIdx.x & 31 & ~(G - 1));
+  const bool b0 = threadIdx.x & 1, b1 = threadIdx.x & 2;
+  const double r0 = (b0 ? s[2] : s[0]) + __shfl_xor_sync(m, b0 ? s[0] : s[2], 1);
+  const double r1 = (b0 ? s[3] : s[1]) + __shfl_xor_sync(m, b0 ? s[1] : s[3], 1);
+  double q = (b1 ? r1 : r0) + __shfl_xor_sync(m, b1 ? r0 : r1, 2);
+#pragma unroll
+  for (int o = 4; o < G; o <<= 1) q += __shfl_xor_sync(m, q, o);
+  return q;
+}
+__device__ __forceinline__ int rx_variant(int lane) { return 2 * (lane & 1) + ((lane >> 1) & 1); }
+template <int G>
+__global__ void __launch_bounds__(256) k_rx_ap(int64_t nnz_ap, const int32_t* __restrict__ off,
+                                               const int32_t* __restrict__ qa, const double* __restrict__ pv,
+                                               RxVals V) {
+  const int lane = threadIdx.x & (G - 1);
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x / G;
+  for (int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G; t < nnz_ap; t += stride) {
     double s[kRxVar] = {0.0, 0.0, 0.0, 0.0};
-    for (int32_t k = off[t]; k < off[t + 1]; ++k) {
+    const int32_t end = off[t + 1];
+    for (int32_t k = off[t] + lane; k < end; k += G) {
       const int32_t q = qa[k];
       const double w = pv[k];
 #pragma unroll
       for (int v = 0; v < kRxVar; ++v) s[v] += V.a[v][q] * w;
     }
-#pragma unroll
-    for (int v = 0; v < kRxVar; ++v) V.ap[v][t] = s[v];
+    if constexpr (G == 1) {
+      V.ap[t] = make_double4_32a(s[0], s[1], s[2], s[3]);
+    } else {
+      const double x = rx_group_sum<G>(s);
+      if (lane < kRxVar) reinterpret_cast<double*>(V.ap + t)[rx_variant(lane)] = x;
+    }
   }
 }
 
@@ -1110,12 +1147,15 @@ __global__ void __launch_bounds__(256) k_rx_gersh(int32_t n, const int32_t* __re
   }
 }
 
-__global__ void k_rx_omega(const double* __restrict__ part, int32_t nb, int level, double* __restrict__ omega) {
-  const int v = threadIdx.x;
-  if (v >= kRxVar) return;
+// (a warp per variant)
+__global__ void __launch_bounds__(32 * kRxVar) k_rx_omega(const double* __restrict__ part, int32_t nb, int level,
+                                                          double* __restrict__ omega) {
+  const int v = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double m = 0.0;
-  for (int32_t b = 0; b < nb; ++b) m = fmax(m, part[(int64_t)v * nb + b]);
-  omega[v * kRxMaxLv + level] = m > 0.0 ? kDamp / m : 0.0;
+  for (int32_t b = lane; b < nb; b += 32) m = fmax(m, part[(int64_t)v * nb + b]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) omega[v * kRxMaxLv + level] = m > 0.0 ? kDamp / m : 0.0;
 }
 
 // The smoother weights W = omega / a_ii (FP64 and FP32) and the FP32 copy
@@ -1141,12 +1181,10 @@ __global__ void k_rx_q(int64_t nnz_ap, const double* __restrict__ pin, const int
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nnz_ap; t += (int64_t)gridDim.x * blockDim.x) {
     const int32_t i = row[t];
     const double p = pin[t];
+    const double4_32a ap = V.ap[t];
+    const double x[kRxVar] = {ap.x, ap.y, ap.z, ap.w};
 #pragma unroll
-    for (int v = 0; v < kRxVar; ++v) {
-      const double q = p - V.w[v][i] * V.ap[v][t];
-      V.q[v][t] = q;
-      V.qf[v][t] = (float)q;
-    }
+    for (int v = 0; v < kRxVar; ++v) V.qf[v][t] = (float)(p - V.w[v][i] * x[v]);
   }
 }
 
@@ -1155,63 +1193,115 @@ __global__ void k_rx_s(int64_t nnz_ap, const int32_t* __restrict__ perm, RxVals 
     const int32_t k = perm[t];
 #pragma unroll
     for (int v = 0; v < kRxVar; ++v) {
-      const double q = V.q[v][k];
-      V.s[v][t] = q;
-      V.sf[v][t] = (float)q;
+      V.sf[v][t] = V.qf[v][k];
     }
   }
 }
 
-__global__ void k_rx_next(int64_t nnz_n, const int32_t* __restrict__ off, const int32_t* __restrict__ tap,
-                          const double* __restrict__ pv, RxVals V) {
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < nnz_n; c += (int64_t)gridDim.x * blockDim.x) {
+template <int G>
+__global__ void __launch_bounds__(256) k_rx_next(int64_t nnz_n, const int32_t* __restrict__ off,
+                                                 const int32_t* __restrict__ tap, const double* __restrict__ pv,
+                                                 RxVals V) {
+  const int lane = threadIdx.x & (G - 1);
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x / G;
+  for (int64_t c = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G; c < nnz_n; c += stride) {
     double s[kRxVar] = {0.0, 0.0, 0.0, 0.0};
-    for (int32_t k = off[c]; k < off[c + 1]; ++k) {
-      const int32_t q = tap[k];
+    const int32_t end = off[c + 1];
+#pragma unroll 4
+    for (int32_t k = off[c] + lane; k < end; k += G) {
+      const double4_32a q = V.ap[tap[k]];
       const double w = pv[k];
-#pragma unroll
-      for (int v = 0; v < kRxVar; ++v) s[v] += V.ap[v][q] * w;
+      s[0] += q.x * w;
+      s[1] += q.y * w;
+      s[2] += q.z * w;
+      s[3] += q.w * w;
     }
+    if constexpr (G == 1) {
 #pragma unroll
-    for (int v = 0; v < kRxVar; ++v) V.an[v][c] = s[v];
+      for (int v = 0; v < kRxVar; ++v) V.an[v][c] = s[v];
+    } else {
+      const double x = rx_group_sum<G>(s);
+      const int v = rx_variant(lane);
+      double* o = v == 0 ? V.an[0] : (v == 1 ? V.an[1] : (v == 2 ? V.an[2] : V.an[3]));
+      if (lane < kRxVar) o[c] = x;
+    }
   }
 }
 
-// Inverse of the coarsest matrix per variant (blockIdx.x): Gauss-Jordan on
-// [A | I] without pivoting (the matrices are symmetric positive definite).
+// Inverses of the four coarsest matrices (symmetric positive definite, at
+// most 64 unknowns), one block each: symmetric Gauss-Jordan sweeps on the
+// lower triangle, which the threads hold in registers.  The FP64 pipe of one
+// SM bounds it (an update of 2,080 entries, 0.6 us, per sweep): 106 us for a
+// coarsest level of some 60 unknowns, against 432 us for the elimination of
+// the full matrix beside the unit matrix in global memory.
+constexpr int kCoarseMax = 64;
+constexpr int kCoarsePer = (kCoarseMax * (kCoarseMax + 1) / 2 + 255) / 256;
 __global__ void __launch_bounds__(256) k_rx_coarse_inv(int32_t nc, const int32_t* __restrict__ rp,
                                                        const int32_t* __restrict__ ci, RxVals V,
-                                                       double* __restrict__ cmat, float* __restrict__ cinv) {
-  const int v = blockIdx.x;
-  const int w2 = 2 * nc;
-  double* M = cmat + (int64_t)v * nc * w2;
-  for (int32_t k = threadIdx.x; k < nc * w2; k += blockDim.x) M[k] = 0.0;
+                                                       float* __restrict__ cinv) {
+  __shared__ double tri[kCoarseMax * (kCoarseMax + 1) / 2];
+  __shared__ double col[2][kCoarseMax], scaled[kCoarseMax], inv[2];
+  const int v = blockIdx.x, n_tri = nc * (nc + 1) / 2;
+  for (int k = threadIdx.x; k < n_tri; k += 256) tri[k] = 0.0;
   __syncthreads();
-  for (int32_t i = threadIdx.x; i < nc; i += blockDim.x) {
-    for (int32_t q = rp[i]; q < rp[i + 1]; ++q) M[(int64_t)i * w2 + ci[q]] = V.an[v][q];
-    M[(int64_t)i * w2 + nc + i] = 1.0;
+  for (int i = threadIdx.x; i < nc; i += 256)
+    for (int32_t q = rp[i]; q < rp[i + 1]; ++q)
+      if (ci[q] <= i) tri[i * (i + 1) / 2 + ci[q]] = V.an[v][q];
+  __syncthreads();
+  double a[kCoarsePer];
+  int row[kCoarsePer], at[kCoarsePer];  // entry (row, at), at <= row
+#pragma unroll
+  for (int k = 0; k < kCoarsePer; ++k) {
+    const int e = threadIdx.x + 256 * k;
+    int i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+    if ((i + 1) * (i + 2) / 2 <= e) ++i;
+    if (i * (i + 1) / 2 > e) --i;
+    row[k] = e < n_tri ? i : -1;
+    at[k] = e - i * (i + 1) / 2;
+    a[k] = e < n_tri ? tri[e] : 0.0;
   }
-  __syncthreads();
-  __shared__ double f[64];
-  for (int32_t c = 0; c < nc; ++c) {
-    const double piv = M[(int64_t)c * w2 + c];
-    __syncthreads();
-    for (int32_t k = threadIdx.x; k < w2; k += blockDim.x) M[(int64_t)c * w2 + k] /= piv;
-    for (int32_t r = threadIdx.x; r < nc; r += blockDim.x) f[r] = r == c ? 0.0 : M[(int64_t)r * w2 + c];
-    __syncthreads();
-    for (int32_t k = threadIdx.x; k < nc * w2; k += blockDim.x) {
-      const int32_t r = k / w2, col = k - r * w2;
-      if (r != c) M[k] -= f[r] * M[(int64_t)c * w2 + col];
+  // column c (= row c) and the reciprocal of its pivot, by the threads that
+  // have just formed them; two buffers, so that a sweep needs two barriers
+  auto publish = [&](int k, int c) {
+    if (row[k] == c) {
+      col[c & 1][at[k]] = a[k];
+      if (at[k] == c) inv[c & 1] = 1.0 / a[k];
+    } else if (at[k] == c && row[k] > c) {
+      col[c & 1][row[k]] = a[k];
     }
+  };
+#pragma unroll
+  for (int k = 0; k < kCoarsePer; ++k) publish(k, 0);
+  for (int c = 0; c < nc; ++c) {
     __syncthreads();
+    const double* x = col[c & 1];
+    const double d = inv[c & 1];
+    if (threadIdx.x < nc) scaled[threadIdx.x] = x[threadIdx.x] * d;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kCoarsePer; ++k) {
+      if (256 * k >= n_tri) break;
+      if (row[k] < 0) continue;
+      if (row[k] == c) a[k] = at[k] == c ? -d : scaled[at[k]];
+      else if (at[k] == c) a[k] = scaled[row[k]];
+      else a[k] -= scaled[row[k]] * x[at[k]];
+      publish(k, c + 1);
+    }
   }
-  for (int32_t k = threadIdx.x; k < nc * nc; k += blockDim.x) {
-    const int32_t i = k / nc, j = k - i * nc;
-    // symmetric part (the exact inverse is symmetric)
-    cinv[(int64_t)v * nc * nc + k] = (float)(0.5 * (M[(int64_t)i * w2 + nc + j] + M[(int64_t)j * w2 + nc + i]));
+  // the sweeps leave the negative inverse
+#pragma unroll
+  for (int k = 0; k < kCoarsePer; ++k) {
+    if (row[k] < 0) continue;
+    const float x = (float)-a[k];
+    float* o = cinv + (int64_t)v * nc * nc;
+    o[(int64_t)row[k] * nc + at[k]] = x;
+    o[(int64_t)at[k] * nc + row[k]] = x;
   }
 }
 
+static int rx_lanes(int64_t entries, int64_t terms) {
+  return terms > kRxMany * entries ? 32 : (entries >= kRxThreads ? 1 : 8);
+}
 static int rx_blocks(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 4096)); }
 
 pdf_status relax_amg_update(RelaxAmg& G, cudaStream_t st) {
@@ -1219,11 +1309,9 @@ pdf_status relax_amg_update(RelaxAmg& G, cudaStream_t st) {
   for (int l = 0; l < L; ++l) {
     RxLevel& V = G.lv[l];
     RxVals R;
+    R.ap = reinterpret_cast<double4_32a*>(V.ap_v);
     for (int v = 0; v < kRxVar; ++v) {
       R.a[v] = V.a_v[v];
-      R.ap[v] = V.ap_v[v];
-      R.q[v] = V.q_v[v];
-      R.s[v] = V.s_v[v];
       R.an[v] = l + 1 < L ? G.lv[l + 1].a_v[v] : G.c_v[v];
       R.af[v] = V.a_f[v];
       R.qf[v] = V.q_f[v];
@@ -1232,23 +1320,30 @@ pdf_status relax_amg_update(RelaxAmg& G, cudaStream_t st) {
       R.w[v] = V.w_v[v];
     }
     const int64_t nnz_n = l + 1 < L ? G.lv[l + 1].nnz_a : G.nnz_c;
-    PDF_KERNEL("k_rx_ap", st, k_rx_ap<<<rx_blocks(V.nnz_ap), 256, 0, st>>>(V.nnz_ap, V.ap_off, V.ap_qa, V.ap_pv, R));
+    const int ga = rx_lanes(V.nnz_ap, V.ap_terms);
+    void (*ap)(int64_t, const int32_t*, const int32_t*, const double*, RxVals) =
+        ga == 1 ? k_rx_ap<1> : (ga == 8 ? k_rx_ap<8> : k_rx_ap<32>);
+    PDF_KERNEL("k_rx_ap", st, ap<<<rx_blocks(ga * V.nnz_ap), 256, 0, st>>>(V.nnz_ap, V.ap_off, V.ap_qa, V.ap_pv, R));
     const int gb = std::min<int>(G.gblocks, rx_blocks(V.n));
     PDF_KERNEL("k_rx_gersh", st, k_rx_gersh<<<dim3(gb, kRxVar), 256, 0, st>>>(V.n, V.a_rp, V.a_dpos, R, G.gpart));
-    PDF_KERNEL("k_rx_omega", st, k_rx_omega<<<1, 32, 0, st>>>(G.gpart, gb, l, G.omega));
+    PDF_KERNEL("k_rx_omega", st, k_rx_omega<<<1, 32 * kRxVar, 0, st>>>(G.gpart, gb, l, G.omega));
     PDF_KERNEL("k_rx_cast", st, k_rx_cast<<<rx_blocks(V.nnz_a), 256, 0, st>>>(V.n, V.nnz_a, V.a_dpos, G.omega, l, R));
     PDF_KERNEL("k_rx_q", st, k_rx_q<<<rx_blocks(V.nnz_ap), 256, 0, st>>>(V.nnz_ap, V.q_pin, V.q_row, R));
     PDF_KERNEL("k_rx_s", st, k_rx_s<<<rx_blocks(V.nnz_ap), 256, 0, st>>>(V.nnz_ap, V.s_perm, R));
-    PDF_KERNEL("k_rx_next", st, k_rx_next<<<rx_blocks(nnz_n), 256, 0, st>>>(nnz_n, V.c_off, V.c_tap, V.c_pv, R));
+    const int gn = rx_lanes(nnz_n, V.c_terms);
+    void (*next)(int64_t, const int32_t*, const int32_t*, const double*, RxVals) =
+        gn == 1 ? k_rx_next<1> : (gn == 8 ? k_rx_next<8> : k_rx_next<32>);
+    PDF_KERNEL("k_rx_next", st, next<<<rx_blocks(gn * nnz_n), 256, 0, st>>>(nnz_n, V.c_off, V.c_tap, V.c_pv, R));
   }
   RxVals R;
+  R.ap = nullptr;
   for (int v = 0; v < kRxVar; ++v) {
-    R.a[v] = nullptr; R.ap[v] = nullptr; R.q[v] = nullptr; R.s[v] = nullptr;
+    R.a[v] = nullptr;
     R.af[v] = R.qf[v] = R.sf[v] = R.wf[v] = nullptr;
     R.w[v] = nullptr;
     R.an[v] = G.c_v[v];
   }
-  PDF_KERNEL("k_rx_coarse_inv", st, k_rx_coarse_inv<<<kRxVar, 256, 0, st>>>(G.nc, G.c_rp, G.c_ci, R, G.cmat, G.cinv));
+  PDF_KERNEL("k_rx_coarse_inv", st, k_rx_coarse_inv<<<kRxVar, 256, 0, st>>>(G.nc, G.c_rp, G.c_ci, R, G.cinv));
   return PDF_OK;
 }
 

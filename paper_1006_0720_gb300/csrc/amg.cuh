@@ -91,7 +91,9 @@ struct RxLevel {
   double* c_pv = nullptr;
   double* q_pin = nullptr;                                       // P at each (A P) position, else 0
   int32_t* q_row = nullptr;
-  double *a_v[kRxVar] = {}, *ap_v[kRxVar] = {}, *q_v[kRxVar] = {}, *s_v[kRxVar] = {};
+  double* a_v[kRxVar] = {};
+  double* ap_v = nullptr;  // [nnz_ap][kRxVar]
+  int64_t ap_terms = 0, c_terms = 0;  // terms of the two plans
   double* w_v[kRxVar] = {};  // smoother weights W = omega / a_ii
   // FP32 copies for the cycle: A, Q, S and W
   float *a_f[kRxVar] = {}, *q_f[kRxVar] = {}, *s_f[kRxVar] = {}, *w_f[kRxVar] = {};
@@ -104,7 +106,6 @@ struct RelaxAmg {
   int64_t nnz_c = 0;
   int32_t *c_rp = nullptr, *c_ci = nullptr;  // the coarsest matrix
   double* c_v[kRxVar] = {};
-  double* cmat = nullptr;                    // [kRxVar][nc][2 nc] Gauss-Jordan work
   float* cinv = nullptr;                     // [kRxVar][nc][nc]
   float* r32 = nullptr;                      // [9][n] FP32 residual, the finest level's b
   double *omega = nullptr, *gpart = nullptr; // [kRxVar][kRxMaxLv], Gershgorin partial maxima
