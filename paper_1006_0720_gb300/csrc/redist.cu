@@ -254,7 +254,7 @@ static int count_bits(int64_t n) {
   return bits;
 }
 
-static pdf_status redist_alloc(pdf_particles* P) {
+static pdf_status redist_alloc(pdf_particles* P, cudaStream_t st) {
   RedistWork& W = P->rd;
   if (W.cnt) return PDF_OK;
   const int64_t nt = P->mesh->d.n_tri;
@@ -268,7 +268,7 @@ static pdf_status redist_alloc(pdf_particles* P) {
   A(&W.v1, nt);
   A(&W.hist, hist_len);
   A(&W.hist_part, radix_part_len());
-  if (e == cudaSuccess) e = cudaMemset(W.hist_part, 0, sizeof(int32_t) * radix_part_len());
+  if (e == cudaSuccess) e = cudaMemsetAsync(W.hist_part, 0, sizeof(int32_t) * radix_part_len(), st);
   A(&W.dev, 4);
   A(&W.role, nt);
   A(&W.cur, 2 * nt);
@@ -290,7 +290,7 @@ extern "C" pdf_status pdf_redistribute(pdf_particles* p, const pdf_mesh* m, int3
   if (!p || !m || p->mesh != m) return fail(PDF_EINVAL, "pdf_redistribute: NULL or mismatched handles");
   if (min_npel < 1 || min_npel > kMaxMin) return fail(PDF_EINVAL, "pdf_redistribute: min_npel must be in [1, 64]");
   cudaStream_t st = (cudaStream_t)stream;
-  pdf_status s = redist_alloc(p);
+  pdf_status s = redist_alloc(p, st);
   if (s != PDF_OK) return s;
   const MeshDev& M = m->d;
   RedistWork& W = p->rd;
