@@ -478,6 +478,11 @@ FX_HD df2 dsub2(df2 a, df2 b) {
 // 2^-56 of what is left.  (The shifts and branches of f2fix, four times per
 // particle, took about three times the instructions.)
 constexpr float kIncMax = 0x1p-23f;
+// Whether an increment lies in that range.  One comparison per part, so that a
+// NaN in any of them is refused (a maximum of two parts drops the NaN).
+FX_HD bool inc_fits(f2 h, f2 l) {
+  return fabsf(h.x) < 1.0f && fabsf(h.y) < 1.0f && fabsf(l.x) <= kIncMax && fabsf(l.y) <= kIncMax;
+}
 FX_HD void add_inc2(int64_t& X, int64_t& Y, f2 h, f2 l) {
   const f2 M1 = dup2(0x1.8p1f), M2 = dup2(0x1.8p-22f), M3 = dup2(0x1.8p-33f);
   const f2 s1 = add2(h, M1);

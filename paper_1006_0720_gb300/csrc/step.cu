@@ -935,10 +935,8 @@ __device__ __forceinline__ bool in_source_fx(const StepArgs& A, const FxArgs& F,
 // Position increment bound of the fixed-point path: |U dt + sqrt(2 nu dt) dW| < 1,
 // which keeps every fixed-point offset of the walk below 2^7, and low parts
 // within the fixed-point sum's range (they exceed it only where two large
-// terms cancel).
-__device__ __forceinline__ bool small_move(const fx::acc2& a) {
-  return fmaxf(fabsf(a.h.x), fabsf(a.h.y)) < 1.0f && fmaxf(fabsf(a.l.x), fabsf(a.l.y)) <= fx::kIncMax;
-}
+// terms cancel).  Increments that are not finite do not pass.
+__device__ __forceinline__ bool small_move(const fx::acc2& a) { return fx::inc_fits(a.h, a.l); }
 
 // FP64 back to the stored forms after the FP64 walk (the wall fall-back).
 __device__ __forceinline__ bool pos_fits(double x) { return fabs(x) < 64.0; }
