@@ -349,11 +349,13 @@ long long prof_launches();
 // blocks of the one before still run; overlap_begin, the first statement of
 // every kernel launched so, waits until all of that kernel's results are
 // visible, then lets the next kernel do the same.  (The wait comes first, so
-// that at most two kernels of a stream are ever resident.)  What a predecessor
-// writes is read through plain pointers (neither __ldg nor __restrict__, whose
-// loads the compiler may move above the wait) unless the address itself comes
-// from a plain load made after the wait.  Nothing changes for a kernel
-// launched in the ordinary way.
+// that at most two kernels of a stream are ever resident.)  What the kernel
+// before writes is read through plain pointers, neither __ldg nor const
+// __restrict__: those loads are for data that no one writes during the
+// kernel's whole life, which begins before the wait.  Mesh tables, and the
+// state arrays in the copy into element order (two kernels behind their
+// writer), may take them.  Nothing changes for a kernel launched in the
+// ordinary way.
 //
 // Blocks that start early go to the SMs that finish early, so a kernel whose
 // one or two waves are bound by work per SM ends later: the passes over the
@@ -381,6 +383,17 @@ inline void launch_over(bool over, void (*kernel)(P...), dim3 grid, unsigned blo
 __device__ __forceinline__ void overlap_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// A load of what the kernel before wrote.  OVER: in a kernel launched over it, a
+// plain load; else the read-only load, which the compiler need not keep behind
+// earlier stores (with plain loads in every kernel 15.9M particles took 11.93
+// instead of 11.82 ms per run of seven steps, 68.6M on the obstacle mesh 35.3
+// instead of 34.5 ms).
+template <bool OVER, typename T>
+__device__ __forceinline__ T ld_result(const T* p) {
+  if constexpr (OVER) return *p;
+  else return __ldg(p);
 }
 
 }  // namespace pdfgb

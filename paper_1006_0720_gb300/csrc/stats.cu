@@ -403,11 +403,15 @@ __global__ void __launch_bounds__(256) k_seg_offsets(const int32_t* keys, int64_
 }
 
 // A stored state value as a double-float (exact for both storage forms).
+template <bool OVER>
 __device__ __forceinline__ fx::df ld_df(const fx::df* a, int64_t i) {
-  const float2 v = __ldg(reinterpret_cast<const float2*>(a) + i);
+  const float2 v = ld_result<OVER>(reinterpret_cast<const float2*>(a) + i);
   return fx::df{v.x, v.y};
 }
-__device__ __forceinline__ fx::df ld_df(const float* a, int64_t i) { return fx::df{__ldg(a + i), 0.f}; }
+template <bool OVER>
+__device__ __forceinline__ fx::df ld_df(const float* a, int64_t i) {
+  return fx::df{ld_result<OVER>(a + i), 0.f};
+}
 
 // Eight lanes per element (four elements per warp), one pass over the
 // element's particles in the grouping's order (sec. 3.3: N, means, central
@@ -499,12 +503,11 @@ __device__ __forceinline__ double moment(const fx::acc (&s1)[5], const fx::acc (
   return __longlong_as_double((long long)fx::df2d(fx::df_norm(fx::mul(fx::sub(pick_acc(s2, m), corr), invN))));
 }
 
-template <typename T>
+template <typename T, bool OVER>
 __global__ void __launch_bounds__(256, 3) k_elem_stats_grp(const int32_t* seg,
-                                                       const int32_t* __restrict__ pid, int32_t n_tri,
-                                                       const T* __restrict__ u, const T* __restrict__ v,
-                                                       const T* __restrict__ w, const T* __restrict__ om,
-                                                       const T* __restrict__ ps, double* __restrict__ es) {
+                                                       const int32_t* pid, int32_t n_tri, const T* u, const T* v,
+                                                       const T* w, const T* om, const T* ps,
+                                                       double* __restrict__ es) {
   overlap_begin();
   const int lane = threadIdx.x & 31, j = lane & (kStatLanes - 1);
   const int64_t group = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kStatLanes;
@@ -533,10 +536,10 @@ __global__ void __launch_bounds__(256, 3) k_elem_stats_grp(const int32_t* seg,
     fx::df2 Kuv{}, Kwp{};
     fx::df Km{0.f, 0.f};
     if (N > 0) {
-      const int32_t p0 = pid ? __ldg(pid + beg) : beg;
-      Kuv = fx::pair(ld_df(u, p0), ld_df(v, p0));
-      Kwp = fx::pair(ld_df(w, p0), ld_df(ps, p0));
-      Km = ld_df(om, p0);
+      const int32_t p0 = pid ? ld_result<OVER>(pid + beg) : beg;
+      Kuv = fx::pair(ld_df<OVER>(u, p0), ld_df<OVER>(v, p0));
+      Kwp = fx::pair(ld_df<OVER>(w, p0), ld_df<OVER>(ps, p0));
+      Km = ld_df<OVER>(om, p0);
     }
     // sums of the deviations (u, v), (w, psi) and of their products (uu, vv),
     // (ww, psi psi), (uw, vw); (uv, the deviations of omega)
@@ -549,7 +552,7 @@ __global__ void __launch_bounds__(256, 3) k_elem_stats_grp(const int32_t* seg,
     // slots loaded one iteration ahead, so that ten state loads are in
     // flight before the first is needed; the sums still take the particles
     // in the lane's order i, i + 8, i + 16, ...
-    auto slot = [&](int32_t i) { return pid ? __ldg(pid + i) : i; };
+    auto slot = [&](int32_t i) { return pid ? ld_result<OVER>(pid + i) : i; };
     int32_t qa = beg + j < end ? slot(beg + j) : 0;
     int32_t qb = beg + j + kStatLanes < end ? slot(beg + j + kStatLanes) : 0;
     auto acc1 = [&](fx::df xu, fx::df xv, fx::df xw, fx::df xm, fx::df xp) {
@@ -570,9 +573,9 @@ __global__ void __launch_bounds__(256, 3) k_elem_stats_grp(const int32_t* seg,
       const bool hb = i + kStatLanes < end;
       qa = i + 2 * kStatLanes < end ? slot(i + 2 * kStatLanes) : 0;
       qb = i + 3 * kStatLanes < end ? slot(i + 3 * kStatLanes) : 0;
-      const fx::df au = ld_df(u, pa), av = ld_df(v, pa), aw = ld_df(w, pa), am = ld_df(om, pa), ap = ld_df(ps, pa);
+      const fx::df au = ld_df<OVER>(u, pa), av = ld_df<OVER>(v, pa), aw = ld_df<OVER>(w, pa), am = ld_df<OVER>(om, pa), ap = ld_df<OVER>(ps, pa);
       fx::df bu = au, bv = av, bw = aw, bm = am, bp = ap;
-      if (hb) { bu = ld_df(u, pb); bv = ld_df(v, pb); bw = ld_df(w, pb); bm = ld_df(om, pb); bp = ld_df(ps, pb); }
+      if (hb) { bu = ld_df<OVER>(u, pb); bv = ld_df<OVER>(v, pb); bw = ld_df<OVER>(w, pb); bm = ld_df<OVER>(om, pb); bp = ld_df<OVER>(ps, pb); }
       acc1(au, av, aw, am, ap);
       if (hb) acc1(bu, bv, bw, bm, bp);
     }
@@ -934,16 +937,18 @@ static pdf_status elem_stats(pdf_particles* P, const int32_t* seg, const int32_t
   // 0.22 ms: with one element per group no group waits for a long one.
   const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)M.n_tri * kStatLanes + 255) / 256,
                                                            (int64_t)sm_count() * 48));
-  if (P->precision == PDF_FP64)
-    PDF_KERNEL("k_elem_stats", st, launch_over(overlap(P->n), k_elem_stats_grp<fx::df>, nb, 256, 0, st, seg, order, M.n_tri,
-               P->u, P->v, P->w, P->om, P->ps, P->es));
-  else
-    PDF_KERNEL("k_elem_stats", st, launch_over(overlap(P->n), k_elem_stats_grp<float>, nb, 256, 0, st, seg, order, M.n_tri,
-               P->uf, P->vf, P->wf, P->omf, P->psf, P->es));
-  return PDF_OK;
+  auto run = [&](auto* u, auto* v, auto* w, auto* om, auto* ps) -> pdf_status {
+    using T = std::remove_reference_t<decltype(*u)>;
+    if (overlap(P->n))
+      PDF_KERNEL("k_elem_stats", st, launch_over(true, k_elem_stats_grp<T, true>, nb, 256, 0, st, seg, order, M.n_tri, u,
+                 v, w, om, ps, P->es));
+    else
+      PDF_KERNEL("k_elem_stats", st, launch_over(false, k_elem_stats_grp<T, false>, nb, 256, 0, st, seg, order, M.n_tri,
+                 u, v, w, om, ps, P->es));
+    return PDF_OK;
+  };
+  return P->precision == PDF_FP64 ? run(P->u, P->v, P->w, P->om, P->ps) : run(P->uf, P->vf, P->wf, P->omf, P->psf);
 }
-
-
 
 // Node statistics and node derivatives from the element statistics P->es
 // (sec. 3.3 second pass, sec. 3.4).

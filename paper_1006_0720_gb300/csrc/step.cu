@@ -511,36 +511,37 @@ struct F32IO {
 // no-slip wall).  The stored forms are widened to FP64 on load and rounded
 // back on store; a particle that is lost, or whose new position leaves
 // |x|, |y| < 64, keeps its position and element.
-template <typename IO>
+template <bool OVER, typename IO>
 __device__ __forceinline__ Counts advance_native(const StepArgs& A, const IO& io, int64_t p, const Draws D) {
   Counts c;
   const float* g = D.g;
   const int32_t e = A.elem[p];
   const double* R = A.rows + (int64_t)e * PDFGB_ROW;
+  auto row = [&](int q) { return ld_result<OVER>(R + q); };
   double U0, U1, U2, o, s;
   io.load(p, U0, U1, U2, o, s);
   const double gx = (double)g[0], gy = (double)g[1];
-  const double d0 = U0 - __ldg(R + 0), d1 = U1 - __ldg(R + 1), d2 = U2 - __ldg(R + 2);
+  const double d0 = U0 - row(0), d1 = U1 - row(1), d2 = U2 - row(2);
   const double G0 = (double)g[2], G1 = (double)g[3], G2 = (double)g[4];
-  const double b = __ldg(R + 21);
+  const double b = row(21);
   // velocity prediction (eq. velocity-prediction), time-n values throughout
-  double un = U0 + __ldg(R + 9) + __ldg(R + 3) * gx + __ldg(R + 4) * gy +
-              __ldg(R + 12) * d0 + __ldg(R + 13) * d1 + __ldg(R + 14) * d2 + b * G0;
-  double vn = U1 + __ldg(R + 10) + __ldg(R + 5) * gx + __ldg(R + 6) * gy +
-              __ldg(R + 15) * d0 + __ldg(R + 16) * d1 + __ldg(R + 17) * d2 + b * G1;
-  double wn = U2 + __ldg(R + 11) + __ldg(R + 7) * gx + __ldg(R + 8) * gy +
-              __ldg(R + 18) * d0 + __ldg(R + 19) * d1 + __ldg(R + 20) * d2 + b * G2;
+  double un = U0 + row(9) + row(3) * gx + row(4) * gy +
+              row(12) * d0 + row(13) * d1 + row(14) * d2 + b * G0;
+  double vn = U1 + row(10) + row(5) * gx + row(6) * gy +
+              row(15) * d0 + row(16) * d1 + row(17) * d2 + b * G1;
+  double wn = U2 + row(11) + row(7) * gx + row(8) * gy +
+              row(18) * d0 + row(19) * d1 + row(20) * d2 + b * G2;
   // position (eq. Lagrangian-position-exact) with the same dW_x, dW_y
   const double x0 = __longlong_as_double((long long)fx::fix2d(A.x[p], kPosF));
   const double y0 = __longlong_as_double((long long)fx::fix2d(A.y[p], kPosF));
   double xn = x0 + U0 * A.dt + A.sdiff * gx;
   double yn = y0 + U1 * A.dt + A.sdiff * gy;
   // frequency (eq. frequency-model); a negative result is reflected
-  double on = o - __ldg(R + 23) * o + __ldg(R + 24) + __ldg(R + 25) * sqrt(fmax(o, 0.0)) * (double)g[5];
+  double on = o - row(23) * o + row(24) + row(25) * sqrt(fmax(o, 0.0)) * (double)g[5];
   if (on < 0.0) { on = -on; ++c.om; }
   // scalar: eq. IEM (element mean) or eq. IECM (the particle's conditional mean)
-  const double tgt = A.cond ? fx::to_double(A.cond[p]) : __ldg(R + 26);
-  const double sn = s - (s - tgt) * __ldg(R + 27);
+  const double tgt = A.cond ? fx::to_double(A.cond[p]) : row(26);
+  const double sn = s - (s - tgt) * row(27);
   // distances from the no-slip wall before and after the move
   const bool near = load_geo(A.geo, e).nsw != 0;
   double dn = 0.0, d1w = 0.0;
@@ -553,12 +554,12 @@ __device__ __forceinline__ Counts advance_native(const StepArgs& A, const IO& io
   const int32_t en = walk(A, e, xn, yn, un, vn, c.walk, c.refl, c.per, c.fb, c.brute, c.near, reinj, wall);
   // no-slip wall condition: trajectory (a) (reflected at a no-slip edge, or
   // behind the wall line) or (b) (eta < f_w, eq. fw): U = 0, omega ~ Gamma
-  if (near && !wall) wall = d1w < 0.0 || wall_eta(A.seed, (uint32_t)__ldg(A.pid + p), A.step) <
+  if (near && !wall) wall = d1w < 0.0 || wall_eta(A.seed, (uint32_t)A.pid[p], A.step) <
                                           exp(-dn * d1w / (A.nu * A.dt));
   if (wall) {
     un = vn = wn = 0.0;
-    const double mw = __ldg(R + 28) > 0.0 ? __ldg(R + 28) : __ldg(R + 22);
-    on = wall_frequency(A.seed, (uint32_t)__ldg(A.pid + p), A.step, mw);
+    const double mw = row(28) > 0.0 ? row(28) : row(22);
+    on = wall_frequency(A.seed, (uint32_t)A.pid[p], A.step, mw);
   }
   if (en >= 0 && fabs(xn) < 64.0 && fabs(yn) < 64.0) {
     A.x[p] = fx::d2fix((uint64_t)__double_as_longlong(xn), kPosF);
@@ -579,11 +580,13 @@ __device__ __forceinline__ Counts advance_native(const StepArgs& A, const IO& io
 // kernel's parameters by reference (they stay in constant memory), all else by
 // value, so that no variable of the caller has its address taken (which would
 // keep it in local memory for its whole life).
+template <bool OVER>
 __device__ __noinline__ Counts advance_native_ool(const StepArgs& A, int64_t p, const Draws D) {
-  return advance_native(A, DfIO{A.u, A.v, A.w, A.om, A.ps}, p, D);
+  return advance_native<OVER>(A, DfIO{A.u, A.v, A.w, A.om, A.ps}, p, D);
 }
+template <bool OVER>
 __device__ __noinline__ Counts advance_native_f32_ool(const StepArgs& A, const F32IO io, int64_t p, const Draws D) {
-  return advance_native(A, io, p, D);
+  return advance_native<OVER>(A, io, p, D);
 }
 
 __device__ __forceinline__ void merge(Counts& a, const Counts& b) {
@@ -602,7 +605,9 @@ __device__ __forceinline__ void flush_counts(const StepArgs& A, const Counts& c)
   add_counter(A.counters + kCntNear, c.near);
 }
 
-__global__ void __launch_bounds__(256) k_step(StepArgs A) {
+// (plain loads of the row without a bound on the registers: 102 instead of 80)
+template <bool OVER>
+__global__ void __launch_bounds__(256, OVER ? 3 : 0) k_step(StepArgs A) {
   overlap_begin();
   Counts c;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -611,7 +616,7 @@ __global__ void __launch_bounds__(256) k_step(StepArgs A) {
   int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   for (int64_t it = 0; it < iters; ++it, p += stride) {
     if (p >= A.n) continue;
-    merge(c, advance_native(A, DfIO{A.u, A.v, A.w, A.om, A.ps}, p, draw_step(A, p)));
+    merge(c, advance_native<OVER>(A, DfIO{A.u, A.v, A.w, A.om, A.ps}, p, draw_step(A, p)));
   }
   flush_counts(A, c);
 }
@@ -649,13 +654,15 @@ struct FxArgs {
   fx::df src_r2;         // r^2
 };
 
+template <bool OVER>
 __device__ __forceinline__ fx::df2 ld_pair(const fx::df2* a) {
-  const float4 v = __ldg(reinterpret_cast<const float4*>(a));
+  const float4 v = ld_result<OVER>(reinterpret_cast<const float4*>(a));
   return fx::df2{fx::f2{v.x, v.y}, fx::f2{v.z, v.w}};
 }
 
+template <bool OVER>
 __device__ __forceinline__ fx::df ld_coef(const fx::df* a) {
-  const float2 v = __ldg(reinterpret_cast<const float2*>(a));
+  const float2 v = ld_result<OVER>(reinterpret_cast<const float2*>(a));
   return fx::df{v.x, v.y};
 }
 
@@ -942,6 +949,7 @@ __device__ __forceinline__ bool small_move(const fx::acc2& a) { return fx::inc_f
 __device__ __forceinline__ bool pos_fits(double x) { return fabs(x) < 64.0; }
 
 
+template <bool OVER>
 __global__ void __launch_bounds__(256, 4) k_step_fx(const __grid_constant__ StepArgs A,
                                                     const __grid_constant__ FxArgs F) {
   overlap_begin();
@@ -991,7 +999,7 @@ __global__ void __launch_bounds__(256, 4) k_step_fx(const __grid_constant__ Step
     const int near_noslip = __ldg(reinterpret_cast<const int*>(F.geo + e) + 18);
     if (!small_move(dxy)) {
       draw_block1(A, id, D);
-      merge(cs, advance_native_ool(A, p, D));
+      merge(cs, advance_native_ool<OVER>(A, p, D));
       continue;
     }
     int64_t Xn = A.x[p], Yn = A.y[p];
@@ -1006,23 +1014,23 @@ __global__ void __launch_bounds__(256, 4) k_step_fx(const __grid_constant__ Step
     // a_i dt starting one each: the pairs are what the row holds and what
     // the draws and differences are, so nothing is moved between lanes.
     const fx::df S = ld_state(A.ps, p);
-    fx::df2 mwp = ld_pair(&R->mean_wp);
+    fx::df2 mwp = ld_pair<OVER>(&R->mean_wp);
     if (A.cond) {  // IECM: the particle's velocity-conditioned mean <phi|V>
       const fx::df cv = ld_state(A.cond, p);
       mwp.h.y = cv.h;
       mwp.l.y = cv.l;
     }
-    const fx::df2 d01 = fx::dsub2(Uuv, ld_pair(&R->mean_uv));
+    const fx::df2 d01 = fx::dsub2(Uuv, ld_pair<OVER>(&R->mean_uv));
     const fx::df2 dwp = fx::dsub2(fx::pair(W, S), mwp);
     const fx::df d2 = dwp.lane0();
     fx::df Un[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       fx::acc2 a;
-      a.init(fx::pair(i == 0 ? Uuv.lane0() : (i == 1 ? Uuv.lane1() : W), ld_coef(&R->a[i])));
-      a.add(fx::mul_f2(ld_pair(&R->grad[i]), g01));
-      a.add(fx::mul_df2(ld_pair(&R->drift[i]), d01));
-      a.add(fx::mul_df2(ld_pair(&R->rest[i]), fx::pair(d2, fx::df{D.g[2 + i], 0.0f})));
+      a.init(fx::pair(i == 0 ? Uuv.lane0() : (i == 1 ? Uuv.lane1() : W), ld_coef<OVER>(&R->a[i])));
+      a.add(fx::mul_f2(ld_pair<OVER>(&R->grad[i]), g01));
+      a.add(fx::mul_df2(ld_pair<OVER>(&R->drift[i]), d01));
+      a.add(fx::mul_df2(ld_pair<OVER>(&R->rest[i]), fx::pair(d2, fx::df{D.g[2 + i], 0.0f})));
       Un[i] = a.fold().value();
     }
     // frequency (eq. frequency-model): omega - (C3 + S_w) <w> dt omega + C3 <w>^2 dt
@@ -1030,9 +1038,9 @@ __global__ void __launch_bounds__(256, 4) k_step_fx(const __grid_constant__ Step
     const fx::df O = ld_state(A.om, p);
     fx::df On;
     {
-      const fx::df2 f = fx::mul_df2(ld_pair(&R->freq), fx::pair(O, fx::sqrt_df(O)));
+      const fx::df2 f = fx::mul_df2(ld_pair<OVER>(&R->freq), fx::pair(O, fx::sqrt_df(O)));
       fx::acc2 a;
-      a.init(fx::pair(O, ld_coef(&R->freq0)));
+      a.init(fx::pair(O, ld_coef<OVER>(&R->freq0)));
       a.add(fx::pair(f.lane0(), fx::mul_f(f.lane1(), D.g[5])));
       On = a.fold().value();
       if (On.h < 0.0f) { On = fx::df{-On.h, -On.l}; ++c_om; }
@@ -1043,11 +1051,11 @@ __global__ void __launch_bounds__(256, 4) k_step_fx(const __grid_constant__ Step
     {
       fx::acc a;
       a.init(S);
-      a.sub(fx::mul(ld_coef(&R->mix), dwp.lane1()));
+      a.sub(fx::mul(ld_coef<OVER>(&R->mix), dwp.lane1()));
       Sn = a.value();
     }
     if (near_noslip) {
-      merge(cs, advance_native_ool(A, p, D));
+      merge(cs, advance_native_ool<OVER>(A, p, D));
       continue;
     }
     // neighbour walk (sec. 3.5) in fixed point; walls, open boundaries and
@@ -1067,8 +1075,8 @@ __global__ void __launch_bounds__(256, 4) k_step_fx(const __grid_constant__ Step
       if (sw.reinj) reinj = true;
       if (sw.noslip) {  // no-slip wall reached through other elements: the wall condition
         const double* Rd = A.rows + (int64_t)A.elem[p] * PDFGB_ROW;
-        const double mw = __ldg(Rd + 28) > 0.0 ? __ldg(Rd + 28) : __ldg(Rd + 22);
-        On = fx::from_double(wall_frequency(A.seed, (uint32_t)__ldg(A.pid + p), A.step, mw));
+        const double mw = Rd[28] > 0.0 ? Rd[28] : Rd[22];
+        On = fx::from_double(wall_frequency(A.seed, (uint32_t)A.pid[p], A.step, mw));
         slow_noslip = true;
       }
       if (sw.e >= 0 && pos_fits(sw.x) && pos_fits(sw.y)) {
@@ -1197,9 +1205,9 @@ __device__ __forceinline__ bool finish_slow(const StepArgs& A, const F32Args& S,
   }
   if (sw.noslip) {  // no-slip wall reached through other elements: the wall condition
     const double* Rd = A.rows + (int64_t)A.elem[p] * PDFGB_ROW;
-    const double mw = __ldg(Rd + 28) > 0.0 ? __ldg(Rd + 28) : __ldg(Rd + 22);
+    const double mw = Rd[28] > 0.0 ? Rd[28] : Rd[22];
     S.u[p] = S.v[p] = S.w[p] = 0.0f;
-    S.om[p] = (float)wall_frequency(A.seed, (uint32_t)__ldg(A.pid + p), A.step, mw);
+    S.om[p] = (float)wall_frequency(A.seed, (uint32_t)A.pid[p], A.step, mw);
   }
   if (sw.e >= 0 && pos_fits(sw.x) && pos_fits(sw.y)) A.elem[p] = sw.e;
   return sw.reinj;
@@ -1237,7 +1245,7 @@ __device__ __noinline__ void queue_run(const StepArgs& A, const FxArgs& F, const
   count_events(Q, c);
 }
 
-template <bool QUEUE>
+template <bool QUEUE, bool OVER>
 __global__ void __launch_bounds__(kStepThreads, 4) k_step_f32(const __grid_constant__ StepArgs A,
                                                               const __grid_constant__ FxArgs F,
                                                               const __grid_constant__ F32Args S) {
@@ -1252,6 +1260,7 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_step_f32(const __grid_const
   auto advance = [&](int64_t p, int64_t& Xn, int64_t& Yn) -> bool {
     const int32_t e = A.elem[p];
     const float* R = S.rows + (int64_t)e * PDFGB_ROW;
+    auto row = [&](int q) { return ld_result<OVER>(R + q); };
     prefetch_l1(R);  // the 128-byte FP32 row and the geometry, as in k_step_fx
     prefetch_l1(F.geo + e);
     if (p + stride < A.n) {
@@ -1268,24 +1277,24 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_step_f32(const __grid_const
     }
     const Draws D = draw_step(A, p);
     const float U0 = S.u[p], U1 = S.v[p], U2 = S.w[p];
-    const float d0 = U0 - __ldg(R + 0), d1 = U1 - __ldg(R + 1), d2 = U2 - __ldg(R + 2);
-    const float b = __ldg(R + 21);
+    const float d0 = U0 - row(0), d1 = U1 - row(1), d2 = U2 - row(2);
+    const float b = row(21);
     // velocity prediction (eq. velocity-prediction) in FP32
-    const float un = U0 + __ldg(R + 9) + __ldg(R + 3) * D.g[0] + __ldg(R + 4) * D.g[1] + __ldg(R + 12) * d0 +
-               __ldg(R + 13) * d1 + __ldg(R + 14) * d2 + b * D.g[2];
-    const float vn = U1 + __ldg(R + 10) + __ldg(R + 5) * D.g[0] + __ldg(R + 6) * D.g[1] + __ldg(R + 15) * d0 +
-               __ldg(R + 16) * d1 + __ldg(R + 17) * d2 + b * D.g[3];
-    const float wn = U2 + __ldg(R + 11) + __ldg(R + 7) * D.g[0] + __ldg(R + 8) * D.g[1] + __ldg(R + 18) * d0 +
-                     __ldg(R + 19) * d1 + __ldg(R + 20) * d2 + b * D.g[4];
+    const float un = U0 + row(9) + row(3) * D.g[0] + row(4) * D.g[1] + row(12) * d0 +
+               row(13) * d1 + row(14) * d2 + b * D.g[2];
+    const float vn = U1 + row(10) + row(5) * D.g[0] + row(6) * D.g[1] + row(15) * d0 +
+               row(16) * d1 + row(17) * d2 + b * D.g[3];
+    const float wn = U2 + row(11) + row(7) * D.g[0] + row(8) * D.g[1] + row(18) * d0 +
+                     row(19) * d1 + row(20) * d2 + b * D.g[4];
     // frequency (eq. frequency-model) and scalar (eq. IEM) in FP32
     const float o = S.om[p];
-    float on = o - __ldg(R + 23) * o + __ldg(R + 24) + __ldg(R + 25) * sqrtf(fmaxf(o, 0.f)) * D.g[5];
+    float on = o - row(23) * o + row(24) + row(25) * sqrtf(fmaxf(o, 0.f)) * D.g[5];
     if (on < 0.f) { on = -on; atomicAdd(&Q.counts[6], 1); }
     const float s = S.ps[p];
-    const float sn = s - (s - (A.cond ? A.cond[p].h : __ldg(R + 26))) * __ldg(R + 27);
+    const float sn = s - (s - (A.cond ? A.cond[p].h : row(26))) * row(27);
     // particles next to a no-slip wall go to the FP64 path
     if (__ldg(reinterpret_cast<const int*>(F.geo + e) + 18) != 0) {
-      count_events(Q, advance_native_f32_ool(A, F32IO{S.u, S.v, S.w, S.om, S.ps}, p, D));
+      count_events(Q, advance_native_f32_ool<OVER>(A, F32IO{S.u, S.v, S.w, S.om, S.ps}, p, D));
       return false;
     }
     // position (eq. Lagrangian-position-exact), fixed point
@@ -1433,26 +1442,32 @@ struct StepLaunch {
   pdf_status run(int64_t beg, int64_t cnt, cudaStream_t st, int per_sm = 16) const {
     if (cnt <= 0) return PDF_OK;
     const int nb = blocks_for(cnt, 256, per_sm);
-    const bool over = cnt <= kOverlapStepMax;
     StepArgs a = A;
     a.n = cnt;
     a.x += beg; a.y += beg; a.elem += beg; a.pid += beg;
     if (a.cond) a.cond += beg;
+    F32Args f = S;
     if (kind == 2) {
-      F32Args f = S;
       f.u += beg; f.v += beg; f.w += beg; f.om += beg; f.ps += beg;
-      // the queue where a warp takes eight rounds or more and fills it; with
-      // fewer the last, partial one is a longer chain than the walk itself
-      if (cnt >= 8 * (int64_t)nb * kStepThreads)
-        PDF_KERNEL("k_step", st, launch_over(over, k_step_f32<true>, nb, kStepThreads, 0, st, a, F, f));
-      else
-        PDF_KERNEL("k_step", st, launch_over(over, k_step_f32<false>, nb, kStepThreads, 0, st, a, F, f));
-    } else if (kind == 1) {
-      a.u += beg; a.v += beg; a.w += beg; a.om += beg; a.ps += beg;
-      PDF_KERNEL("k_step", st, launch_over(over, k_step_fx, nb, 256, 0, st, a, F));
     } else {
       a.u += beg; a.v += beg; a.w += beg; a.om += beg; a.ps += beg;
-      PDF_KERNEL("k_step", st, launch_over(over, k_step, nb, 256, 0, st, a));
+    }
+    return cnt <= kOverlapStepMax ? launch<true>(a, f, nb, st) : launch<false>(a, f, nb, st);
+  }
+
+  template <bool OVER>
+  pdf_status launch(const StepArgs& a, const F32Args& f, int nb, cudaStream_t st) const {
+    if (kind == 2) {
+      // the queue where a warp takes eight rounds or more and fills it; with
+      // fewer the last, partial one is a longer chain than the walk itself
+      if (a.n >= 8 * (int64_t)nb * kStepThreads)
+        PDF_KERNEL("k_step", st, launch_over(OVER, k_step_f32<true, OVER>, nb, kStepThreads, 0, st, a, F, f));
+      else
+        PDF_KERNEL("k_step", st, launch_over(OVER, k_step_f32<false, OVER>, nb, kStepThreads, 0, st, a, F, f));
+    } else if (kind == 1) {
+      PDF_KERNEL("k_step", st, launch_over(OVER, k_step_fx<OVER>, nb, 256, 0, st, a, F));
+    } else {
+      PDF_KERNEL("k_step", st, launch_over(OVER, k_step<OVER>, nb, 256, 0, st, a));
     }
     return PDF_OK;
   }
