@@ -375,8 +375,12 @@ static pdf_status build_levels(HCsr A, int32_t kCoarse, bool with_q, std::vector
   return PDF_OK;
 }
 
-// Pressure systems of at most this many unknowns are solved by one cluster.
-constexpr int32_t kAmgWholeMax = 4096;
+// Pressure systems of at most this many unknowns are solved by one cluster,
+// unless their coarsest system is large: unknowns of the inflow and outflow
+// (rows of the unit matrix) have no couplings and never coarsen, and every CTA
+// of the cluster takes the dense coarsest product for itself.
+constexpr int32_t kAmgWholeMax = 4096, kAmgWholeCoarse = 128;
+static_assert(2 * kAmgWholeCoarse <= kCyShared, "the coarsest vectors fit the shared memory of the levels");
 
 static pdf_status amg_setup_host(int32_t n, const std::vector<int32_t>& rp, const std::vector<int32_t>& ci,
                                  const std::vector<double>& v, bool singular, Amg& G);
@@ -630,7 +634,7 @@ static Cycle<double, 1> amg_cycle(const Amg& G, const double* r, int first, int 
 // component on eight SMs is FP64-bound there).  For the same reason the large
 // form keeps a kernel per sweep on every level: a cluster for the levels
 // below 3,000 unknowns made it 4 % slower.
-bool amg_whole(const Amg& G, int32_t n) { return n <= kAmgWholeMax || G.lv.empty(); }
+bool amg_whole(const Amg& G, int32_t n) { return n <= kAmgWholeMax && G.nc <= kAmgWholeCoarse; }
 
 pdf_status amg_solve(const Amg& G, const AmgSystem& A, int32_t it_end, cudaStream_t st) {
   const int ctas = cy_ctas(A.n);
@@ -659,6 +663,10 @@ pdf_status amg_apply(const Amg& G, const double* r, double* z, double* part, int
     const int32_t nbx = (V.n + 255) / 256, nbc = (int32_t)(((int64_t)V.nc * kG + 255) / 256);
     PDF_KERNEL("k_amg_down", st, k_amg_down<<<nbx + nbc, 256, 0, st>>>(V.n, V.nc, nbx, V.w, V.s_rp, V.s_ci, V.s_v, b,
                                                                         V.x, bc, done));
+  }
+  if (L == 0) {
+    PDF_KERNEL("k_amg_coarse", st, k_amg_coarse<<<(G.nc + 7) / 8, 256, 0, st>>>(G.nc, G.cinv, r, z, done));
+    return PDF_OK;
   }
   PDF_KERNEL("k_amg_coarse", st, k_amg_coarse<<<(G.nc + 7) / 8, 256, 0, st>>>(G.nc, G.cinv, G.cb, G.cz, done));
   for (int32_t l = L - 1; l >= 0; --l) {

@@ -32,10 +32,10 @@ struct Amg {
 pdf_status amg_setup(int32_t n, const std::vector<int32_t>& rp, const std::vector<int32_t>& ci,
                      const std::vector<double>& v, bool singular, Amg& G);
 void amg_free(Amg& G);
-// z = M^-1 r (one V-cycle; a level at least).  The finest up-sweep also
-// forms r . z (block partials in part, finished by the last block through
-// *counter, which it resets): *rz_old = *rz, *rz = r . z.  Every kernel returns
-// at once when *done is set.
+// z = M^-1 r (one V-cycle).  When the hierarchy has a level, the finest
+// up-sweep also forms r . z (block partials in part, finished by the last
+// block through *counter, which it resets): *rz_old = *rz, *rz = r . z;
+// else the caller forms it.  Every kernel returns at once when *done is set.
 pdf_status amg_apply(const Amg& G, const double* r, double* z, double* part, int32_t* counter, double* rz,
                      double* rz_old, const int32_t* done, cudaStream_t st);
 

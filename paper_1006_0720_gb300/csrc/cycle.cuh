@@ -510,6 +510,7 @@ cudaError_t cy_launch(void (*k)(Args...), int clusters, int ctas, size_t shared,
 template <typename T, int V>
 cudaError_t cy_launch_pcg(int comps, int ctas, cudaStream_t st, const CySys<V>& S, const Cycle<T, V>& C,
                           int32_t it_end) {
+  if (2 * (int64_t)C.nc > kCyShared) return cudaErrorInvalidValue;  // (the coarsest vectors, see cy_below)
   const size_t per = ((S.n + ctas - 1) / ctas + 31) & ~31, n = (S.n + 1) & ~1;
   const size_t bytes = sizeof(T) * (kCyShared + 2 * n) + sizeof(double) * (n + 4 * per);
   void (*k)(CySys<V>, Cycle<T, V>, int32_t) = ctas == 1 ? k_cy_pcg<true, T, V> : k_cy_pcg<false, T, V>;

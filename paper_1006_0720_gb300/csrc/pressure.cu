@@ -281,6 +281,30 @@ __global__ void __launch_bounds__(kPBlock) k_press_update(int32_t n_rep, double*
   }
 }
 
+// r . z from its partials when the hierarchy has no level: rz_old = rz,
+// rz = sum.
+__global__ void k_press_rz(const double* __restrict__ part, int32_t nb, double* __restrict__ scal,
+                           const int32_t* __restrict__ done) {
+  if (*done) return;
+  double s = 0.0;
+  for (int32_t i = threadIdx.x; i < nb; i += kPBlock) s += part[i];
+  s = pblock_sum(s);
+  if (threadIdx.x == 0) {
+    scal[kSRzOld] = scal[kSRz];
+    scal[kSRz] = s;
+  }
+}
+
+// r . z partials when the hierarchy has no level (z = the coarse solve).
+__global__ void __launch_bounds__(kPBlock) k_press_dot(int32_t n_rep, const double* __restrict__ r,
+                                                       const double* __restrict__ z, double* __restrict__ part,
+                                                       const int32_t* __restrict__ done) {
+  if (*done) return;
+  const int32_t u = blockIdx.x * kPBlock + threadIdx.x;
+  const double s = pblock_sum(u < n_rep ? r[u] * z[u] : 0.0);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
+}
+
 // partials of sum x (for the zero-mean normalisation)
 __global__ void __launch_bounds__(kPBlock) k_press_xsum(int32_t n_rep, const double* __restrict__ x,
                                                         double* __restrict__ part) {
@@ -602,6 +626,10 @@ static pdf_status press_iterations(PressWork& W, const PressSys& S, int k, cudaS
   for (int i = 0; i < k; ++i) {
     pdf_status s = amg_apply(G, W.r, W.z, W.part, W.ctl + kCtlCount1, W.scal + kSRz, W.scal + kSRzOld, done, st);
     if (s != PDF_OK) return s;
+    if (G.lv.empty()) {
+      PDF_KERNEL("k_press_dot", st, k_press_dot<<<nb, kPBlock, 0, st>>>(S.n, W.r, W.z, W.part, done));
+      PDF_KERNEL("k_press_rz", st, k_press_rz<<<1, kPBlock, 0, st>>>(W.part, nb, W.scal, done));
+    }
     PDF_KERNEL("k_press_dirspmv", st, k_press_dirspmv<<<nb, kPBlock, 0, st>>>(S.n, S.rp, S.ci, S.kmask, W.z, W.p, W.q,
                                                                                W.scal, W.ctl, W.part + nb));
     PDF_KERNEL("k_press_update", st, k_press_update<<<nb, kPBlock, 0, st>>>(S.n, W.scal, W.ctl, W.x, W.r, W.p, W.q,
