@@ -376,11 +376,13 @@ static pdf_status build_levels(HCsr A, int32_t kCoarse, bool with_q, std::vector
 }
 
 // Pressure systems of at most this many unknowns are solved by one cluster,
-// unless their coarsest system is large: unknowns of the inflow and outflow
-// (rows of the unit matrix) have no couplings and never coarsen, and every CTA
-// of the cluster takes the dense coarsest product for itself.
-constexpr int32_t kAmgWholeMax = 4096, kAmgWholeCoarse = 128;
-static_assert(2 * kAmgWholeCoarse <= kCyShared, "the coarsest vectors fit the shared memory of the levels");
+// unless some of them lie on the inflow or outflow.
+constexpr int32_t kAmgWholeMax = 4096;
+// The coarsest system of the kernels per sweep, and the size up to which it is
+// the only one (the dense inverse is the preconditioner, one iteration is
+// enough: 192 unknowns 145 us a call, by levels 335 us).
+constexpr int32_t kAmgDense = 256;
+static_assert(2 * kAmgDense <= kCyShared, "the coarsest vectors fit the shared memory of the levels");
 
 static pdf_status amg_setup_host(int32_t n, const std::vector<int32_t>& rp, const std::vector<int32_t>& ci,
                                  const std::vector<double>& v, bool singular, Amg& G);
@@ -397,9 +399,21 @@ pdf_status amg_setup(int32_t n, const std::vector<int32_t>& rp, const std::vecto
 
 static pdf_status amg_setup_host(int32_t n, const std::vector<int32_t>& rp, const std::vector<int32_t>& ci,
                      const std::vector<double>& v, bool singular, Amg& G) {
-  // (the cluster form takes the dense product in every CTA: at 256 unknowns its
-  // FP64 additions took 18 us per cycle)
-  const int32_t kCoarse = n <= kAmgWholeMax ? 64 : 256;
+  // Unknowns without couplings (rows of the unit matrix: inflow and outflow)
+  // never coarsen.  They come on top of the coarsest size, or levels of little
+  // but them are added in vain (80,000 unknowns with 800 such: six levels and
+  // 8.1 ms a call against four and 3.3 ms), and they keep a system from the
+  // cluster form, where every CTA takes the dense coarsest product for itself
+  // (4,000 unknowns with 200 such: 1.70 ms against 1.08 ms; 40 and fewer:
+  // equal).  In that form 256 coarsest unknowns took 18 us per cycle, so 64.
+  int32_t single = 0;
+  for (int32_t i = 0; i < n; ++i) {
+    bool coupled = false;
+    for (int32_t q = rp[i]; q < rp[i + 1]; ++q) coupled = coupled || (ci[q] != i && v[q] != 0.0);
+    single += !coupled;
+  }
+  const bool whole = n <= kAmgDense || (n <= kAmgWholeMax && single == 0);
+  const int32_t kCoarse = whole && n > kAmgDense ? 64 : kAmgDense + single;
   HCsr A0;
   A0.n = A0.m = n;
   A0.rp = rp;
@@ -467,6 +481,7 @@ static pdf_status amg_setup_host(int32_t n, const std::vector<int32_t>& rp, cons
     s = dev_vec(&L.x, L.n);
   }
   G.nc = nc;
+  G.whole = whole && nc <= kAmgDense;
   if (s == PDF_OK) s = up(&G.cinv, Inv);
   if (s == PDF_OK) s = dev_vec(&G.cb, nc);
   if (s == PDF_OK) s = dev_vec(&G.cz, nc);
@@ -634,8 +649,6 @@ static Cycle<double, 1> amg_cycle(const Amg& G, const double* r, int first, int 
 // component on eight SMs is FP64-bound there).  For the same reason the large
 // form keeps a kernel per sweep on every level: a cluster for the levels
 // below 3,000 unknowns made it 4 % slower.
-bool amg_whole(const Amg& G, int32_t n) { return n <= kAmgWholeMax && G.nc <= kAmgWholeCoarse; }
-
 pdf_status amg_solve(const Amg& G, const AmgSystem& A, int32_t it_end, cudaStream_t st) {
   const int ctas = cy_ctas(A.n);
   CySys<1> S;

@@ -24,6 +24,7 @@ struct Amg {
   int32_t nc = 0;           // coarsest size
   double* cinv = nullptr;   // [nc][nc] regularised inverse of the coarsest matrix
   double *cb = nullptr, *cz = nullptr;
+  bool whole = false;       // solved by one cluster in one launch (amg_solve)
 };
 
 // Builds the hierarchy of the symmetric CSR matrix (n rows, columns
@@ -41,7 +42,7 @@ pdf_status amg_apply(const Amg& G, const double* r, double* z, double* part, int
 
 // The whole preconditioned conjugate-gradient solve of a system of n
 // unknowns by one cluster in one launch, up to iteration it_end (*done = 1 at
-// r.r <= *tol2 or a breakdown); amg_whole: whether a system takes this form.
+// r.r <= *tol2 or a breakdown), for hierarchies with G.whole.
 struct AmgSystem {
   int32_t n = 0;
   const int32_t *rp = nullptr, *ci = nullptr;
@@ -49,7 +50,6 @@ struct AmgSystem {
   double *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *rr = nullptr, *rz = nullptr, *tol2 = nullptr;
   int32_t *iters = nullptr, *done = nullptr;
 };
-bool amg_whole(const Amg& G, int32_t n);
 pdf_status amg_solve(const Amg& G, const AmgSystem& A, int32_t it_end, cudaStream_t st);
 
 // The whole preconditioned conjugate-gradient iteration for the CSR matrix

@@ -722,7 +722,7 @@ extern "C" pdf_status pdf_pressure_project(pdf_particles* p, const pdf_mesh* m, 
   }
   if (coop) {
     // nothing else to launch
-  } else if (amg_whole(*S.amg, S.n)) {
+  } else if (S.amg->whole) {
     // launches of at most 1,024 iterations, so that no launch runs for long
     // when the residual stalls above the threshold
     AmgSystem A;
