@@ -337,6 +337,11 @@ pdf_status host_io_stage(pdf_particles* p, int64_t cap);
 // Launches through prof_launch are counted and, when timing is enabled,
 // bracketed by CUDA events on the launch stream.
 void prof_launch(const char* name, cudaStream_t st, void (*launch)(void*), void* ctx);
+// Set-up work (uploads from pageable memory, cleared arrays) goes to the legacy
+// stream, and a non-blocking stream does not wait for that one: every set-up
+// ends by waiting for it, so that the caller's stream may use the results.
+inline cudaError_t setup_wait() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 // Whether per-kernel timing is on; adding launches made by a graph replay
 // to the counter; the counter itself.
 bool prof_timing();

@@ -433,6 +433,11 @@ extern "C" pdf_status pdf_mesh_create(const double* node_xy, int32_t n_nodes, co
     if (t != PDF_TAG_INFLOW && t != PDF_TAG_OUTFLOW) continue;
     for (int q = 0; q < 2; ++q) m->inout[bnd_edge[3 * i + q]] = t == PDF_TAG_INFLOW ? 1 : 2;
   }
+  const cudaError_t e = setup_wait();
+  if (e != cudaSuccess) {
+    pdf_mesh_destroy(m);
+    return cuda_fail(e, "pdf_mesh_create");
+  }
   *out = m;
   return PDF_OK;
 }

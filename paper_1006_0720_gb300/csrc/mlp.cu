@@ -677,6 +677,8 @@ extern "C" pdf_status pdf_mlp_params(pdf_mlp* M, const float* set, float* get, c
   if (set) {
     PDF_KERNEL("k_mlp_pack", (cudaStream_t)0, k_mlp_pack<<<(kNWb + 255) / 256, 256>>>(M->w, M->wb, M->bias));
     PDF_CUDA(cudaDeviceSynchronize());
+  } else if (set_norm) {
+    PDF_CUDA(setup_wait());
   }
   return PDF_OK;
 }

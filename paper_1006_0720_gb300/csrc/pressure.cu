@@ -443,6 +443,7 @@ static pdf_status press_alloc(pdf_particles* P) {
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&W.cs, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&W.ev0, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&W.ev1, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = setup_wait();
   if (e != cudaSuccess) {
     press_free(W);
     return cuda_fail(e, "pdf_pressure_project: allocation");
@@ -601,6 +602,7 @@ static pdf_status sys_get(pdf_particles* P, int k, PressSys** out) {
       cudaError_t e = cudaMalloc((void**)&S.gw, sizeof(double) * std::max(S.n, 1));
       if (e == cudaSuccess) e = cudaMalloc((void**)&S.gw_prev, sizeof(double) * std::max(S.n, 1));
       if (e == cudaSuccess) e = cudaMemset(S.gw_prev, 0, sizeof(double) * std::max(S.n, 1));
+      if (e == cudaSuccess) e = setup_wait();
       if (e != cudaSuccess) s = cuda_fail(e, "pdf_pressure_project: allocation");
     }
     if (s != PDF_OK) {

@@ -419,6 +419,7 @@ static pdf_status relax_amg_build(pdf_particles* P) {
     return PDF_OK;
   }
   W.amg = G;
+  PDF_CUDA(setup_wait());
   return PDF_OK;
 }
 
@@ -451,6 +452,7 @@ static pdf_status relax_alloc(pdf_particles* P) {
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&W.cs, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&W.ev0, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&W.ev1, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = setup_wait();
   if (e != cudaSuccess) {
     relax_free(W);
     return cuda_fail(e, "pdf_relax_solve: allocation");
