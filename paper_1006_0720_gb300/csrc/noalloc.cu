@@ -1,6 +1,6 @@
 // pdf_estimate_stats_noalloc: the statistics entry point for callers that
 // must not allocate device memory.  The grouping scratch (radix keys and
-// values, tile histograms, scan partials, segment offsets) lives in one
+// values, tile histograms, segment offsets) lives in one
 // file-scope device array instead of buffers from cudaMalloc.
 #include <mutex>
 
@@ -9,7 +9,7 @@
 namespace pdfgb {
 pdf_status estimate_stats_with_buffers(pdf_particles* P, int32_t* keys_a, int32_t* vals_a,
                                        int32_t* keys_b, int32_t* vals_b, int32_t* hist,
-                                       int32_t* hist_part, int32_t* seg, cudaStream_t st);
+                                       int64_t hist_len, int32_t* seg, cudaStream_t st);
 }  // namespace pdfgb
 
 using namespace pdfgb;
@@ -20,11 +20,10 @@ constexpr int64_t kMaxParticles = PDF_NOALLOC_MAX_PARTICLES;  // 2^19
 constexpr int64_t kMaxElements = PDF_NOALLOC_MAX_ELEMENTS;    // 2^18
 constexpr int64_t kMaxTiles = (kMaxParticles + 4095) / 4096;  // radix tiles of 4096 keys
 constexpr int64_t kHistInts = kMaxTiles * 512;
-constexpr int64_t kPartInts = 520;  // the digit totals of the scan (512), rounded up
-// int32 layout: keys_a | vals_a | keys_b | vals_b | hist | part | seg
-constexpr int64_t kScratchInts = 4 * kMaxParticles + kHistInts + kPartInts + (kMaxElements + 1);
+// int32 layout: keys_a | vals_a | keys_b | vals_b | hist | seg
+constexpr int64_t kScratchInts = 4 * kMaxParticles + kHistInts + (kMaxElements + 1);
 
-// 4 x 2 MiB + 256 KiB + 2 KiB + 1 MiB: every GPU that loads the library
+// 4 x 2 MiB + 256 KiB + 1 MiB: every GPU that loads the library
 // holds these ~9.2 MiB until the process exits.
 static __device__ __align__(256) int32_t g_noalloc_scratch[kScratchInts];
 
@@ -65,12 +64,12 @@ extern "C" pdf_status pdf_estimate_stats_noalloc(pdf_particles* p, const pdf_mes
   int32_t* keys_b = vals_a + kMaxParticles;
   int32_t* vals_b = keys_b + kMaxParticles;
   int32_t* hist = vals_b + kMaxParticles;
-  int32_t* part = hist + kHistInts;
-  int32_t* seg = part + kPartInts;
+  int32_t* seg = hist + kHistInts;
   cudaStream_t st = (cudaStream_t)stream;
   // Nothing in the scratch has to start at zero: every pass writes all the
-  // histogram entries, scan partials and key/value slots it later reads.
-  pdf_status s = estimate_stats_with_buffers(p, keys_a, vals_a, keys_b, vals_b, hist, part, seg, st);
+  // histogram entries and key/value slots it later reads, and the scatter sums
+  // the tile counts itself (a scan would need sums that start at zero).
+  pdf_status s = estimate_stats_with_buffers(p, keys_a, vals_a, keys_b, vals_b, hist, kHistInts, seg, st);
   if (s != PDF_OK) return s;
   const MeshDev& M = m->d;
   if (elem_stats)

@@ -1015,18 +1015,22 @@ namespace pdfgb {
 
 // Statistics with caller-chosen grouping buffers (used by the
 // allocation-free entry point in noalloc.cu).  keys_b/vals_b receive the
-// result; at most two passes of 9-bit digits, so n_tri <= 2^18; hist holds
-// 512 entries per 4,096 keys, and the tile counts are never scanned (at most
-// 128 tiles).
+// result; at most two passes of 9-bit digits, so n_tri <= 2^18, and at most
+// kFusedTiles tiles, so that no pass scans (there is no space for a scan's
+// sums); hist holds hist_len entries.
+static_assert((PDF_NOALLOC_MAX_PARTICLES + kTileLarge - 1) / kTileLarge <= kFusedTiles,
+              "the largest set without allocations is grouped without a scan");
+static_assert(PDF_NOALLOC_MAX_ELEMENTS <= 1 << 18, "two digits of 9 bits");
 pdf_status estimate_stats_with_buffers(pdf_particles* P, int32_t* keys_a, int32_t* vals_a,
                                        int32_t* keys_b, int32_t* vals_b, int32_t* hist,
-                                       int32_t* hist_part, int32_t* seg, cudaStream_t st) {
+                                       int64_t hist_len, int32_t* seg, cudaStream_t st) {
   const MeshDev& M = P->mesh->d;
   const RadixPlan R = radix_plan(P->n, key_bits_of(M.n_tri), 9);
-  if (R.passes > 2) return fail(PDF_EINVAL, "estimate_stats_with_buffers: more than 2^18 elements");
+  if (R.passes > 2 || !R.fused || (R.tiles << R.bits) > hist_len)
+    return fail(PDF_EINVAL, "estimate_stats_with_buffers: the grouping's plan does not fit the buffers");
   int32_t* const kout[2] = {R.passes == 2 ? keys_a : keys_b, keys_b};
   int32_t* const vout[2] = {R.passes == 2 ? vals_a : vals_b, vals_b};
-  pdf_status s = group_keys(R, P->elem, P->n, M.n_tri, hist, hist_part, kout, vout, seg, st);
+  pdf_status s = group_keys(R, P->elem, P->n, M.n_tri, hist, nullptr, kout, vout, seg, st);
   if (s != PDF_OK) return s;
   const int32_t* vin = vals_b;
   s = elem_stats(P, seg, vin, st);
