@@ -661,7 +661,7 @@ pdf_status amg_solve(const Amg& G, const AmgSystem& A, int32_t it_end, cudaStrea
   S.on = 0; S.off = 1;
   const Cycle<double, 1> C = amg_cycle(G, nullptr, 0, ctas);
   cudaError_t e = cudaSuccess;
-  PDF_KERNEL("k_press_pcg", st, e = (cy_launch_pcg<double, 1>(1, ctas, st, S, C, it_end)));
+  PDF_KERNEL("k_press_pcg", st, e = (cy_launch_pcg<kAmgWholeMax, double, 1>(1, ctas, st, S, C, it_end)));
   return e == cudaSuccess ? PDF_OK : cuda_fail(e, "k_press_pcg");
 }
 

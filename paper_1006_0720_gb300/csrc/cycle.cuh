@@ -507,14 +507,27 @@ cudaError_t cy_launch(void (*k)(Args...), int clusters, int ctas, size_t shared,
   return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
-template <typename T, int V>
+// Dynamic shared memory of k_cy_pcg for n unknowns on clusters of `ctas` CTAs.
+template <typename T>
+constexpr size_t cy_pcg_shared(int64_t n, int64_t ctas) {
+  const size_t per = (size_t)(((n + ctas - 1) / ctas + 31) & ~31), ns = (size_t)((n + 1) & ~1);
+  return sizeof(T) * (kCyShared + 2 * ns) + sizeof(double) * (ns + 4 * per);
+}
+
+// MAX_N: the most unknowns the caller solves so.  A kernel's limit of dynamic
+// shared memory belongs to the kernel, not to the launch, and handles of several
+// threads share it: every call sets the same one, that of the largest system
+// (a limit per size was lowered by one thread between another's setting and
+// its launch).
+template <int32_t MAX_N, typename T, int V>
 cudaError_t cy_launch_pcg(int comps, int ctas, cudaStream_t st, const CySys<V>& S, const Cycle<T, V>& C,
                           int32_t it_end) {
-  if (2 * (int64_t)C.nc > kCyShared) return cudaErrorInvalidValue;  // (the coarsest vectors, see cy_below)
-  const size_t per = ((S.n + ctas - 1) / ctas + 31) & ~31, n = (S.n + 1) & ~1;
-  const size_t bytes = sizeof(T) * (kCyShared + 2 * n) + sizeof(double) * (n + 4 * per);
+  // up to 256 unknowns one CTA, 256 per CTA below eight of them
+  const size_t limit = ctas == 1 ? cy_pcg_shared<T>(256, 1) : cy_pcg_shared<T>(MAX_N, kCyMaxCtas);
+  const size_t bytes = cy_pcg_shared<T>(S.n, ctas);
+  if (bytes > limit || 2 * (int64_t)C.nc > kCyShared) return cudaErrorInvalidValue;  // (the latter: see cy_below)
   void (*k)(CySys<V>, Cycle<T, V>, int32_t) = ctas == 1 ? k_cy_pcg<true, T, V> : k_cy_pcg<false, T, V>;
-  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
   return e == cudaSuccess ? cy_launch(k, comps, ctas, bytes, st, S, C, it_end) : e;
 }
 

@@ -447,7 +447,7 @@ pdf_status relax_mg_solve(const RelaxAmg& G, const RxSystem& A, int32_t it_end, 
   S.on = 1; S.off = 0;
   const RxCycle C = make_cycle(G, 0, ctas);
   cudaError_t e = cudaSuccess;
-  PDF_KERNEL("k_rx_pcg", st, e = (cy_launch_pcg<float, kRxVar>(9, ctas, st, S, C, it_end)));
+  PDF_KERNEL("k_rx_pcg", st, e = (cy_launch_pcg<kWholeMax, float, kRxVar>(9, ctas, st, S, C, it_end)));
   return e == cudaSuccess ? PDF_OK : cuda_fail(e, "k_rx_pcg");
 }
 
