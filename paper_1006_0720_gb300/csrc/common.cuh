@@ -355,8 +355,8 @@ long long prof_launches();
 // every kernel launched so, waits until all of that kernel's results are
 // visible, then lets the next kernel do the same.  (The wait comes first, so
 // that at most two kernels of a stream are ever resident.)  What the kernel
-// before writes is read through plain pointers, neither __ldg nor const
-// __restrict__: those loads are for data that no one writes during the
+// before writes is read through plain pointers (or ld_result), neither __ldg
+// nor const __restrict__: those loads are for data that no one writes during the
 // kernel's whole life, which begins before the wait.  Mesh tables, and the
 // state arrays in the copy into element order (two kernels behind their
 // writer), may take them.  Nothing changes for a kernel launched in the
@@ -367,9 +367,13 @@ long long prof_launches();
 // nodes and elements overlap only on small meshes (79,600 nodes: a run's
 // statistics 0.3 ms longer with it), the particle kernel up to two million
 // particles (5.1M: 1 % slower), the others up to eight million (68.6M: 1 %
-// slower).  Runs of seven steps: 74,100 particles 0.84 -> 0.69 ms, 411,000
+// slower).  The element statistics have a block per 32 elements, each as long
+// as its elements are full, so few blocks of full elements crowd on a few
+// SMs: they overlap up to 256 particles per element (in no order, 400 on 1,482
+// elements: 92 us without, 156 us with, 119 us before either form; 300 on 870:
+// 73 and 71 us).  Runs of seven steps: 74,100 particles 0.84 -> 0.69 ms, 411,000
 // 1.20 -> 1.02 ms, 5.1M 4.00 -> 3.88 ms.
-constexpr int64_t kOverlapMax = 8000000, kOverlapStepMax = 2000000;
+constexpr int64_t kOverlapMax = 8000000, kOverlapStepMax = 2000000, kOverlapPpe = 256;
 inline bool overlap(int64_t n) { return n <= kOverlapMax; }
 template <typename... P, typename... A>
 inline void launch_over(bool over, void (*kernel)(P...), dim3 grid, unsigned block, size_t shared, cudaStream_t st, A... args) {
@@ -390,14 +394,42 @@ __device__ __forceinline__ void overlap_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// A load of what the kernel before wrote.  OVER: in a kernel launched over it, a
-// plain load; else the read-only load, which the compiler need not keep behind
-// earlier stores (with plain loads in every kernel 15.9M particles took 11.93
-// instead of 11.82 ms per run of seven steps, 68.6M on the obstacle mesh 35.3
-// instead of 34.5 ms).
+// A load of what the kernel before wrote and this one leaves as it is, from an
+// address that comes from a plain load made after the wait.  OVER: in a kernel
+// launched over it, an ordinary global load that the compiler may schedule like
+// arithmetic; the address keeps it behind the wait.  Else the read-only load.
+// (Plain loads stay behind every store before them and cost more: with them
+// in every kernel 15.9M particles took 11.93 instead of 11.82 ms per run of
+// seven steps; FP32 statistics of 522,000 particles on 870 elements 76 us,
+// with these 69 us.)
+__device__ __forceinline__ float ld_global(const float* p) {
+  float v;
+  asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld_global(const double* p) {
+  double v;
+  asm("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int32_t ld_global(const int32_t* p) {
+  int32_t v;
+  asm("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float2 ld_global(const float2* p) {
+  float2 v;
+  asm("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_global(const float4* p) {
+  float4 v;
+  asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
 template <bool OVER, typename T>
 __device__ __forceinline__ T ld_result(const T* p) {
-  if constexpr (OVER) return *p;
+  if constexpr (OVER) return ld_global(p);
   else return __ldg(p);
 }
 

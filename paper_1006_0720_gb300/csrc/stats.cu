@@ -939,7 +939,7 @@ static pdf_status elem_stats(pdf_particles* P, const int32_t* seg, const int32_t
                                                            (int64_t)sm_count() * 48));
   auto run = [&](auto* u, auto* v, auto* w, auto* om, auto* ps) -> pdf_status {
     using T = std::remove_reference_t<decltype(*u)>;
-    if (overlap(P->n))
+    if (overlap(P->n) && P->n <= kOverlapPpe * M.n_tri)
       PDF_KERNEL("k_elem_stats", st, launch_over(true, k_elem_stats_grp<T, true>, nb, 256, 0, st, seg, order, M.n_tri, u,
                  v, w, om, ps, P->es));
     else
