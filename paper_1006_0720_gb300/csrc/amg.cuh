@@ -98,6 +98,7 @@ struct RxLevel {
   // FP32 copies for the cycle: A, Q, S and W
   float *a_f[kRxVar] = {}, *q_f[kRxVar] = {}, *s_f[kRxVar] = {}, *w_f[kRxVar] = {};
   float *b = nullptr, *x = nullptr, *z = nullptr;                // [9][n] (b, z for l > 0; level 0's b is r32)
+  char* mem = nullptr;  // the allocation of the arrays from a_v on (A P too)
 };
 
 struct RelaxAmg {
