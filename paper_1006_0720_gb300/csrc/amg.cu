@@ -1045,7 +1045,7 @@ static pdf_status relax_amg_setup_host(int32_t n, const std::vector<int32_t>& rp
         (s = up_vec(&L.q_pin, q_pin)) != PDF_OK || (s = up_vec(&L.q_row, q_row)) != PDF_OK)
       break;
     // the values and vectors, cleared, in one allocation (one each per array made
-    // the first solve on 6,300 nodes 3 % longer than the solve it replaced)
+    // the first solve on 3,200 nodes 12.5 -> 13.3 ms)
     size_t bytes = 0;
     auto place = [&](auto** p, int64_t n) {  // (an offset until the base is known)
       *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(bytes);

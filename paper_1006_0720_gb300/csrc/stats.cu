@@ -64,19 +64,21 @@ int64_t radix_hist_len(int64_t n, int key_bits) {
 constexpr int kScanChunks = 64;  // of tiles
 int32_t radix_part_len() { return (1 + kScanChunks) << kMaxBits; }  // and the chunk sums of the scan
 
-// Per-tile digit histogram, tile by tile: hist[tile * bins + digit].  (Digit by
-// digit, every count went to a sector of its own: with 10-bit digits the
-// 32-byte sectors of a tile's counts were twice the bytes of its keys, here
-// and again in the scatter.)  Thread t counts the tile's keys PER t ... PER (t + 1) - 1 (16-byte loads when the keys are 16-byte aligned)
-// as runs of equal digits, one shared atomic per run: the element ids arrive
-// nearly sorted (the state is reordered by element every few steps, and the
-// second pass reads the first pass's output), so a thread's keys are mostly
-// one or two runs.  sums (zero before, or NULL): the counts of each chunk of tiles,
-// [kScanChunks][bins], for k_scan_bins.
-// Tiles of chunk c: [n_tiles c / 64, n_tiles (c + 1) / 64); the chunk of a tile.
+// The chunk of a tile: chunk c holds the tiles [n_tiles c / 64, n_tiles (c + 1) / 64).
 __device__ __forceinline__ int64_t scan_chunk(int64_t n_tiles, int64_t tile) {
   return (kScanChunks * (tile + 1) - 1) / n_tiles;
 }
+
+// Per-tile digit histogram, tile by tile: hist[tile * bins + digit].  (Digit by
+// digit, every count went to a sector of its own: with 10-bit digits the
+// 32-byte sectors of a tile's counts were twice the bytes of its keys, here
+// and again in the scatter.)  Thread t counts the tile's keys PER t ... PER (t + 1) - 1
+// (16-byte loads when the keys are 16-byte aligned) as runs of equal digits,
+// one shared atomic per run: the element ids arrive nearly sorted (the state
+// is reordered by element every few steps, and the second pass reads the first
+// pass's output), so a thread's keys are mostly one or two runs.  sums (zero
+// before, or NULL): the counts of each chunk of tiles, [kScanChunks][bins], for
+// k_scan_bins.
 template <int BITS, int TILE>
 __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const int32_t* keys, int64_t n,
                                                              int shift, int sub, int32_t* __restrict__ hist,
